@@ -68,7 +68,7 @@ struct di_ctx {
     // workspace capacity
     int cap_w = 0, cap_h = 0, cap_c = 0;
     void* pool = nullptr;           // one allocation for every level buffer
-    float* planes = nullptr;        // 4 * C * n0 floats
+    float* parked = nullptr;        // oras_scratch_floats (null if none)
     double* partials = nullptr;     // residual norm partial sums
     size_t partials_cap = 0;
     double* norm2 = nullptr;        // [kMaxChannels]
@@ -229,10 +229,10 @@ void free_workspace(di_ctx* ctx) {
         ctx->cg[k] = nullptr;
     }
     if (ctx->pool) cudaFree(ctx->pool);
-    if (ctx->planes) cudaFree(ctx->planes);
+    if (ctx->parked) cudaFree(ctx->parked);
     if (ctx->partials) cudaFree(ctx->partials);
     ctx->pool = nullptr;
-    ctx->planes = nullptr;
+    ctx->parked = nullptr;
     ctx->partials = nullptr;
     ctx->partials_cap = 0;
     ctx->cap_w = ctx->cap_h = ctx->cap_c = 0;
@@ -269,9 +269,10 @@ di_status ensure_workspace(di_ctx* ctx, int w, int h, int C) {
     const int L = num_levels(nw, nh, ctx->cfg.block);
     cudaError_t e = cudaMalloc(&ctx->pool, pool_bytes(nw, nh, nc, L, ctx->cfg.precision));
     if (e != cudaSuccess) { ctx->pool = nullptr; return cuda_fail(ctx, e, "cudaMalloc(pool)"); }
-    e = cudaMalloc(&ctx->planes,
-                   oras_scratch_floats(nw, nh, nc, ctx->cfg.block, ctx->cfg.overlap) * sizeof(float));
-    if (e != cudaSuccess) { free_workspace(ctx); return cuda_fail(ctx, e, "cudaMalloc(planes)"); }
+    if (const size_t np = oras_scratch_floats(nw, nh, nc, ctx->cfg.block, ctx->cfg.overlap)) {
+        e = cudaMalloc(&ctx->parked, np * sizeof(float));
+        if (e != cudaSuccess) { free_workspace(ctx); return cuda_fail(ctx, e, "cudaMalloc(parked)"); }
+    }
     ctx->partials_cap = residual_partials_per_channel(nw, nh) * nc;
     e = cudaMalloc(&ctx->partials, ctx->partials_cap * sizeof(double));
     if (e != cudaSuccess) { free_workspace(ctx); return cuda_fail(ctx, e, "cudaMalloc(partials)"); }
@@ -392,7 +393,7 @@ struct Sched {
         }
         DI_CUDA(ctx, launch_oras(in, zero_in, rhs, rhs_zero, v.mbits, v.w, v.h, C, ctx->cfg.block,
                                  ctx->cfg.overlap, ctx->cfg.alpha, iters, rtol2, out,
-                                 ctx->planes, maxupd, s, ev, ctx->cfg.precision,
+                                 ctx->parked, maxupd, s, ev, ctx->cfg.precision,
                                  ctx->upd + kMaxUpdSlots,
                                  l == 0 && ctx->cfg.profile ? ctx->dsteps : nullptr, stor(l),
                                  f64(l), pro_e, pro_max, pro_mode));
@@ -1466,7 +1467,7 @@ di_status di_oras_iteration(di_ctx* ctx, const float* u_in, const float* b, int 
     DI_CUDA(ctx, launch_pack_mask(c, width, height, bits, nullptr, s));
     DI_CUDA(ctx, launch_oras(u_in, 0, b, rhs_zero ? 1 : 0, bits, width, height, channels,
                              ctx->cfg.block, ctx->cfg.overlap, ctx->cfg.alpha, local_iters, 0.f,
-                             u_out, ctx->planes, nullptr, s, nullptr, ctx->cfg.precision,
+                             u_out, ctx->parked, nullptr, s, nullptr, ctx->cfg.precision,
                              ctx->upd + kMaxUpdSlots, nullptr, kF32,
                              ctx->cfg.refine_fp64 != 0));
     return DI_OK;
@@ -1496,7 +1497,7 @@ di_status di_prolong_oras_iteration(di_ctx* ctx, const float* uH, int mode, cons
     DI_CUDA(ctx, launch_pack_mask(c, width, height, bits, nullptr, s));
     DI_CUDA(ctx, launch_oras(u_in, 0, b, rhs_zero ? 1 : 0, bits, width, height, channels, 32,
                              ctx->cfg.overlap, ctx->cfg.alpha, local_iters, 0.f, u_out,
-                             ctx->planes, nullptr, s, nullptr, ctx->cfg.precision,
+                             ctx->parked, nullptr, s, nullptr, ctx->cfg.precision,
                              ctx->upd + kMaxUpdSlots, nullptr, kF32, ctx->cfg.refine_fp64 != 0,
                              uH, nullptr, mode));
     return DI_OK;

@@ -93,15 +93,15 @@ cudaError_t launch_pyramid_level(const uint8_t* c, const float* b, int w, int h,
 cudaError_t launch_pack_mask(const uint8_t* c, int w, int h, uint32_t* bits,
                              unsigned long long* unknown, cudaStream_t s);
 
-// Floats of ORAS scratch for an image of w x h x C: four parity planes of
-// pixels shared along y, then the compact strips of pixels shared along x only.
+// Floats of ORAS scratch for an image of w x h x C: where blocks share pixels
+// (overlap 1 or >= 3), one BxB tile of weighted contributions per block and
+// channel.
 inline size_t oras_scratch_floats(int w, int h, int C, int B, int o) {
-    const int nsh = o == 1 ? 1 : (o > 2 ? o - 2 : 0);
-    const int nbx = axis_blocks_decl(w, B, o);
-    return 4 * (size_t)w * h * C + 2 * (size_t)C * (nbx > 1 ? nbx - 1 : 0) * h * (nsh > 0 ? nsh : 1);
+    if (o == 2) return 0;
+    return (size_t)axis_blocks_decl(w, B, o) * axis_blocks_decl(h, B, o) * C * B * B;
 }
 
-// One ORAS iteration u_in -> u_out (planes: oras_scratch_floats of workspace;
+// One ORAS iteration u_in -> u_out (parked: oras_scratch_floats of workspace;
 // mbits: the packed mask of this level).  Each local CG runs `iters` steps or
 // until r.r <= max(rtol2, 1e-14) * (r.r)_0 (rtol2 >= 0), or until
 // r.r <= max(1e-14 (r.r)_0, -rtol2) (rtol2 < 0: an absolute level, per block
@@ -123,7 +123,7 @@ inline size_t oras_scratch_floats(int w, int h, int C, int B, int o) {
 // (the cascade's interpolation, u_in = b); only where prolong_fusable() holds.
 cudaError_t launch_oras(const float* u_in, int zero_in, const float* rhs, int rhs_zero,
                         const uint32_t* mbits, int w, int h, int C, int B, int o, float alpha,
-                        int iters, float rtol2, float* u_out, float* planes, unsigned* maxupd,
+                        int iters, float rtol2, float* u_out, float* parked, unsigned* maxupd,
                         cudaStream_t s, cudaEvent_t* ev = nullptr, int precision = 0,
                         unsigned* errflag = nullptr, unsigned long long* step_count = nullptr,
                         int stor = kF32, bool f64 = false, const float* pro_e = nullptr,

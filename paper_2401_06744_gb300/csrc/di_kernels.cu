@@ -21,9 +21,8 @@
 //                    TMA; optionally the start formed by prolongation inside it
 //   k_oras_2w_h      the same with FP16 / BF16 local iterates
 //   k_oras_warp      8x8 and 16x16 blocks: one warp per (block, channel)
-//   k_combine_rows/cols  Algorithm 2 step 3 for pixels shared by several
-//                    blocks: sum the weighted block contributions in a fixed
-//                    order (shared rows full width, then shared columns)
+//   k_combine        Algorithm 2 step 3 for pixels shared by several blocks: the
+//                    sums of their weighted contributions in a fixed order
 //   k_plan, k_stop   the device-driven decode: levels in use and start, and the
 //                    stop test after every V-cycle (conditional graph nodes)
 //   k_batch_*        the batched form: the same steps over the segment tables of
@@ -32,10 +31,10 @@
 //
 // Layout: images planar [C][h][w] float32, masks [h][w] uint8.  The ORAS
 // block pass writes pixels that only one block weights (weight 1) straight to
-// u_out and parks weighted contributions of shared pixels in four parity
-// planes [4][C][h][w] (blocks with equal (kx & 1, ky & 1) never overlap, so
-// every plane pixel has one writer); the combine pass adds them in a fixed
-// order, which keeps the result deterministic without atomics.
+// u_out and parks weighted contributions of shared pixels in a BxB tile of its
+// own per block and channel ([block][channel][B][B], so every word has one
+// writer); the combine pass adds them in a fixed order, which keeps the result
+// deterministic without atomics.
 #include "di_internal.h"
 #include "../../include/di.h"
 
@@ -102,33 +101,6 @@ template <> __device__ __forceinline__ void stf<float>(float* p, float v) { *p =
 template <> __device__ __forceinline__ void stf<__half>(__half* p, float v) { *p = __float2half_rn(v); }
 template <> __device__ __forceinline__ void stf<__nv_bfloat16>(__nv_bfloat16* p, float v) {
     *p = __float2bfloat16_rn(v);
-}
-
-// Block index k = min(g / s, nb - 1) without an integer division: a float
-// estimate from the reciprocal, corrected by one step either way.
-__device__ __forceinline__ int block_of(int g, int s, float inv_s, int nb) {
-    int k = __float2int_rd(((float)g + 0.5f) * inv_s);
-    if (k * s > g) --k;
-    else if ((k + 1) * s <= g) ++k;
-    return k > nb - 1 ? nb - 1 : k;
-}
-
-// Blocks with nonzero weight at global coordinate g along one axis: returns
-// 1 (k0) or 2 (k0 < k1).
-__device__ __forceinline__ int axis_contrib(int g, int s, int o, int nb, int& k0, int& k1,
-                                            float inv_s) {
-    const int k = block_of(g, s, inv_s, nb);
-    const int j = g - k * s;
-    k1 = k;
-    if (k > 0 && j < o) {
-        if (o == 1) { k0 = k - 1; return 2; }
-        if (j == 0) { k0 = k - 1; return 1; }
-        if (j == o - 1) { k0 = k; return 1; }
-        k0 = k - 1;
-        return 2;
-    }
-    k0 = k;
-    return 1;
 }
 
 // ---------------------------------------------------------------------------
@@ -1008,7 +980,7 @@ __global__ void __launch_bounds__(32)
 k_oras_warp(const float* __restrict__ u_in, int zero_in, const float* __restrict__ rhs,
             int rhs_zero, const uint32_t* __restrict__ mbits, int wpr, int w, int h, int C,
             int o, int nbx, int nby, float alpha, int iters, float rtol2,
-            float* __restrict__ u_out, float* __restrict__ planes, unsigned* __restrict__ maxupd,
+            float* __restrict__ u_out, float* __restrict__ parked, unsigned* __restrict__ maxupd,
             int chan_inner, unsigned long long* __restrict__ step_count) {
     using WT = WarpTile<B>;
     constexpr int G = WT::G, R = WT::R, NP = WT::NP, TH = WT::TH, P = WT::P, TILE = WT::TILE;
@@ -1237,24 +1209,13 @@ k_oras_warp(const float* __restrict__ u_in, int zero_in, const float* __restrict
             ++nsteps;
         }
 
-        // u_out = u_in + sum_i R_i^T D_i v_i: weight-1 pixels directly, shared
-        // pixels through the parity planes.
-        // x-only shared pixels go to the compact seam strips that follow the
-        // four parity planes: strip[side][ch][seam - 1][y][j], side 0 = left block
+        // u_out = u_in + sum_i R_i^T D_i v_i: weight-1 pixels directly, the
+        // weighted part of shared pixels parked in the block's tile for k_combine
+        // (the first contributor of a shared pixel, smallest block index along
+        // each shared axis, also carries u_in, so the combine pass only adds)
         const int nsh = shared_per_seam(o), first = shared_first(o);
-        int sx_seam = -1, sx_side = 0, sx_j = 0;
-        if (kx > 0 && col >= first && col < first + nsh) {
-            sx_seam = kx; sx_side = 1; sx_j = col - first;
-        } else if (kx < nbx - 1 && col - s >= first && col - s < first + nsh) {
-            sx_seam = kx + 1; sx_side = 0; sx_j = col - s - first;
-        }
-        float* strip = sx_seam > 0
-                           ? planes + 4 * (size_t)C * n +
-                                 (((size_t)(sx_side * C + ch) * (nbx - 1) + (sx_seam - 1)) * h) *
-                                     nsh + sx_j
-                           : planes;
-        const int par = (kx & 1) | ((ky & 1) << 1);
-        float* plane = planes + ((size_t)par * C + ch) * n;
+        const bool xfirst = !(kx > 0 && col >= first && col < first + nsh);
+        float* mine = parked + ((size_t)blk * C + ch) * (B * B) + col;
         float* uo = u_out + ch * n;
         const bool colok = x0 + col < w;
 #pragma unroll
@@ -1265,22 +1226,12 @@ k_oras_warp(const float* __restrict__ u_in, int zero_in, const float* __restrict
                 if (ly >= bh || !colok) continue;
                 const float v = e ? hi2(x[k]) : lo2(x[k]);
                 const float d = wx * s_wy[ly];
-                const size_t gp = (size_t)(y0 + ly) * w + x0 + col;
-                // the first contributor of a shared pixel (smallest block
-                // index along each shared axis) also carries u_in, so the
-                // combine passes only add parked values
                 const float uold = zero_in ? 0.f : tu[(ly + 1) * P + col + 1];
                 if (d == 1.f) {
-                    uo[gp] = uold + v;
+                    uo[(size_t)(y0 + ly) * w + x0 + col] = uold + v;
                 } else if (d > 0.f) {
-                    const float wyr = s_wy[ly];
-                    const bool xfirst = sx_seam < 0 || sx_side == 0;  // no left partner on x
-                    if (wyr < 1.f) {
-                        const bool yfirst = ly >= s;  // upper block of its row overlap
-                        plane[gp] = (xfirst && yfirst) ? uold + d * v : d * v;
-                    } else {
-                        strip[(size_t)(y0 + ly) * nsh] = xfirst ? uold + d * v : d * v;
-                    }
+                    const bool yfirst = !(ky > 0 && ly >= first && ly < first + nsh);
+                    mine[ly * B] = (xfirst && yfirst) ? uold + d * v : d * v;
                 }
                 if (d > 0.f) vmax = fmaxf(vmax, fabsf(v));
             }
@@ -1485,14 +1436,15 @@ __device__ __forceinline__ void tma_load_3d(unsigned dst, const CUtensorMap* map
 // the known pixels and P eH at the unknown ones (prolong_body's mode 0 with
 // u_in as b: the cascade's interpolation of the coarser level's solution).
 // Each block forms the start in its tile (block pixels and halo) before the
-// residual.  Needs u_in (not zero_in) and an even block stride, so that the
+// residual.  SHARED: blocks share pixels (overlap 1 or >= 3); otherwise
+// (overlap 2) the partition weights are 0 and 1.  Needs u_in (not zero_in) and an even block stride, so that the
 // parity of a block pixel is that of its tile index.
-template <bool F64, int PRO>
+template <bool F64, int PRO, bool SHARED>
 __global__ void __launch_bounds__(64, 8)
 k_oras_2w(const float* __restrict__ u_in, int zero_in, const float* __restrict__ rhs,
           int rhs_zero, const uint32_t* __restrict__ mbits, int wpr, int w, int h, int C, int o,
           int nbx, int nby, float alpha, int iters, float rtol2, float* __restrict__ u_out,
-          float* __restrict__ planes, unsigned* __restrict__ maxupd, int chan_inner,
+          float* __restrict__ parked, unsigned* __restrict__ maxupd, int chan_inner,
           const __grid_constant__ CUtensorMap tm_u, const __grid_constant__ CUtensorMap tm_b,
           int use_tma, unsigned* __restrict__ errflag,
           unsigned long long* __restrict__ step_count, const float* __restrict__ eH, int wH,
@@ -1865,10 +1817,9 @@ k_oras_2w(const float* __restrict__ u_in, int zero_in, const float* __restrict__
             ++nsteps;
         }
 
-        const int nsh = shared_per_seam(o);
         float* uo = u_out + ch * n;
         const bool colok = x0 + col < w;
-        if (nsh == 0) {
+        if constexpr (!SHARED) {
             // 0/1 weights (overlap 2): each pixel is written by the one block
             // whose weight is 1 there, with u_in added
             if (colok && wx > 0.f) {
@@ -1887,21 +1838,13 @@ k_oras_2w(const float* __restrict__ u_in, int zero_in, const float* __restrict__
                 }
             }
         } else {
-            // x-only shared pixels go to the compact seam strips that follow the
-            // four parity planes: strip[side][ch][seam - 1][y][j], side 0 = left block
-            const int first = shared_first(o);
-            int sx_seam = -1, sx_side = 0, sx_j = 0;
-            if (kx > 0 && col >= first && col < first + nsh) {
-                sx_seam = kx; sx_side = 1; sx_j = col - first;
-            } else if (kx < nbx - 1 && col - s >= first && col - s < first + nsh) {
-                sx_seam = kx + 1; sx_side = 0; sx_j = col - s - first;
-            }
-            const size_t strip_row0 =
-                ((size_t)(sx_side * C + ch) * (nbx - 1) + (sx_seam - 1)) * h;
-            float* strip = sx_seam > 0 ? planes + 4 * (size_t)C * n + strip_row0 * nsh + sx_j
-                                       : planes;
-            const int par = (kx & 1) | ((ky & 1) << 1);
-            float* plane = planes + ((size_t)par * C + ch) * n;
+            // the weighted part of shared pixels is parked in the block's tile
+            // for k_combine; the first contributor of a shared pixel (smallest
+            // block index along each shared axis) also carries u_in, so the
+            // combine pass only adds
+            const int first = shared_first(o), nsh = shared_per_seam(o);
+            const bool xfirst = !(kx > 0 && col >= first && col < first + nsh);
+            float* const mine = parked + ((size_t)blk * C + ch) * (B * B) + col;
 #pragma unroll
             for (int k = 0; k < NP; ++k) {
 #pragma unroll
@@ -1910,22 +1853,12 @@ k_oras_2w(const float* __restrict__ u_in, int zero_in, const float* __restrict__
                     if (ly >= bh || !colok) continue;
                     const float v = e ? hi2(x[k]) : lo2(x[k]);
                     const float d = wx * s_wy[ly];
-                    const size_t gp = (size_t)(y0 + ly) * w + x0 + col;
-                    // the first contributor of a shared pixel (smallest block
-                    // index along each shared axis) also carries u_in, so the
-                    // combine passes only add parked values
                     const float uold = zero_in ? 0.f : tu[(ly + 1) * P + col + 1];
                     if (d == 1.f) {
-                        uo[gp] = uold + v;
+                        uo[(size_t)(y0 + ly) * w + x0 + col] = uold + v;
                     } else if (d > 0.f) {
-                        const float wyr = s_wy[ly];
-                        const bool xfirst = sx_seam < 0 || sx_side == 0;  // no left partner on x
-                        if (wyr < 1.f) {
-                            const bool yfirst = ly >= s;  // upper block of its row overlap
-                            plane[gp] = (xfirst && yfirst) ? uold + d * v : d * v;
-                        } else {
-                            strip[(size_t)(y0 + ly) * nsh] = xfirst ? uold + d * v : d * v;
-                        }
+                        const bool yfirst = !(ky > 0 && ly >= first && ly < first + nsh);
+                        mine[ly * B] = (xfirst && yfirst) ? uold + d * v : d * v;
                     }
                     if (d > 0.f) vmax = fmaxf(vmax, fabsf(v));
                 }
@@ -1989,7 +1922,7 @@ __global__ void __launch_bounds__(64, 10)
 k_oras_2w_h(const TU* __restrict__ u_in, int zero_in, const TU* __restrict__ rhs,
             int rhs_zero, const uint32_t* __restrict__ mbits, int wpr, int w, int h, int C, int o,
             int nbx, int nby, float alpha, int iters, float rtol2, TU* __restrict__ u_out,
-            float* __restrict__ planes, unsigned* __restrict__ maxupd, int chan_inner,
+            float* __restrict__ parked, unsigned* __restrict__ maxupd, int chan_inner,
             unsigned long long* __restrict__ step_count) {
     constexpr bool kAsync = std::is_same<TU, float>::value;
     typedef typename H::T2 T2;
@@ -2256,22 +2189,11 @@ k_oras_2w_h(const TU* __restrict__ u_in, int zero_in, const TU* __restrict__ rhs
             ++nsteps;
         }
 
-        const int par = (kx & 1) | ((ky & 1) << 1);
-        float* plane = planes + ((size_t)par * C + ch) * n;
         TU* uo = u_out + ch * n;
         const bool colok = x0 + col < w;
         const int nsh = shared_per_seam(o), first = shared_first(o);
-        int sx_seam = -1, sx_side = 0, sx_j = 0;
-        if (kx > 0 && col >= first && col < first + nsh) {
-            sx_seam = kx; sx_side = 1; sx_j = col - first;
-        } else if (kx < nbx - 1 && col - s >= first && col - s < first + nsh) {
-            sx_seam = kx + 1; sx_side = 0; sx_j = col - s - first;
-        }
-        float* strip = sx_seam > 0
-                           ? planes + 4 * (size_t)C * n +
-                                 (((size_t)(sx_side * C + ch) * (nbx - 1) + (sx_seam - 1)) * h) *
-                                     nsh + sx_j
-                           : planes;
+        const bool xfirst = !(kx > 0 && col >= first && col < first + nsh);
+        float* const mine = parked + ((size_t)blk * C + ch) * (B * B) + col;
         const float vs = bad ? 0.f : sc;  // a non-finite narrow iterate gives no correction
 #pragma unroll
         for (int k = 0; k < NP; ++k) {
@@ -2281,19 +2203,12 @@ k_oras_2w_h(const TU* __restrict__ u_in, int zero_in, const TU* __restrict__ rhs
                 if (ly >= bh || !colok) continue;
                 const float v = (e ? H::hi(x[k]) : H::lo(x[k])) * vs;
                 const float d = wx * s_wy[ly];
-                const size_t gp = (size_t)(y0 + ly) * w + x0 + col;
                 const float uold = zero_in ? 0.f : tu[(ly + 1) * P + col + 1];
                 if (d == 1.f) {
-                    stf(uo + gp, uold + v);
+                    stf(uo + (size_t)(y0 + ly) * w + x0 + col, uold + v);
                 } else if (d > 0.f) {
-                    const float wyr = s_wy[ly];
-                    const bool xfirst = sx_seam < 0 || sx_side == 0;
-                    if (wyr < 1.f) {
-                        const bool yfirst = ly >= s;
-                        plane[gp] = (xfirst && yfirst) ? uold + d * v : d * v;
-                    } else {
-                        strip[(size_t)(y0 + ly) * nsh] = xfirst ? uold + d * v : d * v;
-                    }
+                    const bool yfirst = !(ky > 0 && ly >= first && ly < first + nsh);
+                    mine[ly * B] = (xfirst && yfirst) ? uold + d * v : d * v;
                 }
                 if (d > 0.f) vmax = fmaxf(vmax, fabsf(v));
             }
@@ -2310,59 +2225,66 @@ k_oras_2w_h(const TU* __restrict__ u_in, int zero_in, const TU* __restrict__ rhs
     }
 }
 
-// Shared rows (the interior rows of every horizontal overlap), full width:
-// contributions from the parity planes (two block rows; two block columns
-// where the pixel is also shared along x).
-template <class TU>
+// The sums of the pixels that several blocks share (overlap 1 or >= 3), in the
+// fixed order upper left, upper right, lower left, lower right; the first term
+// carries u_in.  A warp takes one part of a (block, channel): blockIdx.z = 0 the
+// seam left of the block (two blocks), 1 the seam above it (two), 2 the corner
+// where they cross (four).  One launch per iteration instead of a row and a
+// column pass: with the parts in tiles by block, a warp reaches all its
+// addresses from one block index.  Bound by latency (one dependent load round
+// trip per warp, four rows in flight), not bytes: that is why the parts go to
+// three warps instead of one after the other.  At overlap 6 an ORAS iteration
+// on 1920x1080 RGB went from 116 to 107 us, a decode of that size from 1.38 to
+// 1.20 ms and one of 481x321 RGB from 1.05 to 0.91 ms (one warp for all three
+// parts: 1.22 ms and no gain at 481x321).
+template <class TU, int B>
 __global__ void __launch_bounds__(256)
-k_combine_rows(const float* __restrict__ planes,
-               int w, int h, int s, int o, int nbx, int nby, float inv_s,
-               TU* __restrict__ u_out) {
-    const int x = blockIdx.x * blockDim.x + threadIdx.x;
-    const int ch = blockIdx.z, C = gridDim.z;
-    if (x >= w) return;
-    const int nsh = shared_per_seam(o);
-    const int seam = blockIdx.y / nsh + 1;             // lower block row of the overlap
-    const int y = seam * s + shared_first(o) + (int)blockIdx.y % nsh;
-    if (y >= h) return;
-    int kx0, kx1;
-    const int nx = axis_contrib(x, s, o, nbx, kx0, kx1, inv_s);
-    const size_t n = (size_t)w * h, gp = (size_t)y * w + x;
-    const size_t cs = (size_t)C * n;
-    const float* pl = planes + ch * n + gp;
-    const int pu = (seam - 1) & 1, pdn = seam & 1;  // y parity of the upper / lower block
-    // the first term (upper-left block) already carries u_in
-    float acc = pl[(size_t)((kx0 & 1) | (pu << 1)) * cs];
-    if (nx == 2) acc += pl[(size_t)((kx1 & 1) | (pu << 1)) * cs];
-    acc += pl[(size_t)((kx0 & 1) | (pdn << 1)) * cs];
-    if (nx == 2) acc += pl[(size_t)((kx1 & 1) | (pdn << 1)) * cs];
-    stf(u_out + ch * n + gp, acc);
-}
-
-// Pixels shared along x only: thread (j, row) adds the strip entries of the
-// left and right block for pixel j of the seam's shared run in that row (j
-// fastest, so the strip reads of a warp are contiguous).
-template <class TU>
-__global__ void __launch_bounds__(256)
-k_combine_cols(const float* __restrict__ planes,
-               int w, int h, int s, int o, int nbx, int nby, float inv_s,
-               TU* __restrict__ u_out) {
-    const int j = threadIdx.x;
-    const int y = blockIdx.x * blockDim.y + threadIdx.y;
-    const int seam = (int)blockIdx.y + 1;
-    const int ch = blockIdx.z, C = gridDim.z;
-    if (y >= h) return;
-    const int x = seam * s + shared_first(o) + j;
-    if (x >= w) return;
-    int ky0, ky1;
-    if (axis_contrib(y, s, o, nby, ky0, ky1, inv_s) == 2) return;  // shared row: k_combine_rows
-    const int nsh = shared_per_seam(o);
-    const size_t n = (size_t)w * h;
-    const float* strips = planes + 4 * (size_t)C * n;
-    const size_t side = (size_t)C * (nbx - 1) * h * nsh;
-    const size_t at = (((size_t)ch * (nbx - 1) + (seam - 1)) * h + y) * nsh + j;
-    // the left block's entry already carries u_in
-    stf(u_out + ch * n + (size_t)y * w + x, strips[at] + strips[at + side]);
+k_combine(const float* __restrict__ parked, int w, int h, int C, int o, int nbx, int nby,
+          TU* __restrict__ u_out) {
+    const int lane = threadIdx.x & 31;
+    const int unit = (int)blockIdx.x * 8 + (int)(threadIdx.x >> 5);  // kx * C + ch
+    if (unit >= nbx * C) return;
+    const int kx = unit / C, ch = unit - kx * C, ky = blockIdx.y;
+    const int s = B - o, x0 = kx * s, y0 = ky * s;
+    const int nsh = shared_per_seam(o), first = shared_first(o);
+    // lanes over the shared run of a seam: j < nsh of the next power of two
+    const int js = nsh > 8 ? 4 : nsh > 4 ? 3 : nsh > 2 ? 2 : nsh > 1 ? 1 : 0;
+    const int j = lane & ((1 << js) - 1), i0 = lane >> js, di = 32 >> js;
+    // rows / columns of the block that only the seam's own blocks weight
+    const int wlo = o == 1 ? 1 : o - 1, whi = o == 1 ? s - 1 : s;
+    TU* dst = u_out + ((size_t)ch * h + y0) * w + x0;
+    const float* me = parked + ((size_t)ky * nbx * C + unit) * (B * B);
+    const float* lf = me - (size_t)C * (B * B) + s;            // left block, from its column s
+    const float* up = me - (size_t)nbx * C * (B * B) + s * B;  // upper block, from its row s
+    // rows i, i + step, ... <= hi of column x: the sum of two tiles, four rows in flight
+    auto add2_rows = [&](const float* a, int i, int hi, int step, int x) {
+        for (; i <= hi; i += 4 * step) {
+            float v[4];
+#pragma unroll
+            for (int m = 0; m < 4; ++m) {
+                const int r = i + m * step;
+                v[m] = r <= hi ? a[r * B + x] + me[r * B + x] : 0.f;
+            }
+#pragma unroll
+            for (int m = 0; m < 4; ++m)
+                if (i + m * step <= hi) stf(dst + (size_t)(i + m * step) * w + x, v[m]);
+        }
+    };
+    if (blockIdx.z == 0) {
+        if (kx > 0 && j < nsh)
+            add2_rows(lf, (ky > 0 ? wlo : 0) + i0, ky < nby - 1 ? whi : min(B, h - y0) - 1, di,
+                      first + j);
+    } else if (blockIdx.z == 1) {
+        const int x = lane & (B - 1);
+        if (ky > 0 && x >= (kx > 0 ? wlo : 0) && x <= (kx < nbx - 1 ? whi : min(B, w - x0) - 1))
+            add2_rows(up, first + lane / B, first + nsh - 1, 32 / B, x);
+    } else if (kx > 0 && ky > 0 && j < nsh) {
+        const float* ul = up - (size_t)C * (B * B) + s;
+        const int x = first + j;
+        for (int i = first + i0; i < first + nsh; i += di)
+            stf(dst + (size_t)i * w + x,
+                ul[i * B + x] + up[i * B + x] + lf[i * B + x] + me[i * B + x]);
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -3016,7 +2938,8 @@ inline dim3 grid2(int w, int h, dim3 blk, int z = 1) {
                 (unsigned)z);
 }
 
-cudaError_t launch_combine(float* planes, int w, int h, int C, int B, int o, int nbx, int nby,
+template <int B>
+cudaError_t launch_combine(const float* parked, int w, int h, int C, int o, int nbx, int nby,
                            float* u_out, cudaStream_t s, int stor);
 
 // cuTensorMapEncodeTiled from the driver, looked up once through the runtime
@@ -3099,12 +3022,12 @@ template <class H, class TU, bool F64>
 void run_oras_2w_h(int grid, size_t smem, cudaStream_t s, const float* u_in, int zero_in,
                    const float* rhs, int rhs_zero, const uint32_t* mbits, int wpr, int w, int h,
                    int C, int o, int nbx, int nby, float alpha, int iters, float rtol2,
-                   float* u_out, float* planes, unsigned* maxupd, int chan_inner,
+                   float* u_out, float* parked, unsigned* maxupd, int chan_inner,
                    unsigned long long* step_count) {
     k_oras_2w_h<H, TU, F64><<<grid, 64, smem, s>>>(
         reinterpret_cast<const TU*>(u_in), zero_in, reinterpret_cast<const TU*>(rhs), rhs_zero,
         mbits, wpr, w, h, C, o, nbx, nby, alpha, iters, rtol2, reinterpret_cast<TU*>(u_out),
-        planes, maxupd, chan_inner, step_count);
+        parked, maxupd, chan_inner, step_count);
 }
 
 template <class H, class TU, bool F64>
@@ -3120,7 +3043,7 @@ const void* oras_2w_h_fn() {
 // |P e| of mode 1 into *pro_max.
 cudaError_t launch_oras_2w(const float* u_in, int zero_in, const float* rhs, int rhs_zero,
                            const uint32_t* mbits, int wpr, int w, int h, int C, int o, float alpha,
-                           int iters, float rtol2, float* u_out, float* planes, unsigned* maxupd,
+                           int iters, float rtol2, float* u_out, float* parked, unsigned* maxupd,
                            cudaStream_t s, cudaEvent_t* ev, int precision, unsigned* errflag,
                            unsigned long long* step_count, int stor, bool f64,
                            const float* pro_e, unsigned* pro_max, int pro_mode) {
@@ -3137,6 +3060,7 @@ cudaError_t launch_oras_2w(const float* u_in, int zero_in, const float* rhs, int
     int nsm = 0, oc = 0;
     size_t smem = 0;
     const void* kern = nullptr;
+    decltype(&k_oras_2w<false, 0, false>) fn = nullptr;  // the FP32 kernel
     CUtensorMap tm_u, tm_b, tm_e;
     std::memset(&tm_u, 0, sizeof tm_u);
     std::memset(&tm_b, 0, sizeof tm_b);
@@ -3149,9 +3073,13 @@ cudaError_t launch_oras_2w(const float* u_in, int zero_in, const float* rhs, int
         use_tma_e = use_tma && pm != 0 &&
                     make_map(&tm_e, pro_e, wH, hH, C, Smem2W::EPW, Smem2W::EH);
         smem = Smem2W::bytes(!rhs_zero, pm != 0);
-        kern = pm == 1 ? (f64 ? (const void*)k_oras_2w<true, 1> : (const void*)k_oras_2w<false, 1>)
-               : pm == 2 ? (f64 ? (const void*)k_oras_2w<true, 2> : (const void*)k_oras_2w<false, 2>)
-                         : (f64 ? (const void*)k_oras_2w<true, 0> : (const void*)k_oras_2w<false, 0>);
+#define DI_ORAS_SEL(SH)                                                                \
+    (pm == 1   ? (f64 ? k_oras_2w<true, 1, SH> : k_oras_2w<false, 1, SH>)               \
+     : pm == 2 ? (f64 ? k_oras_2w<true, 2, SH> : k_oras_2w<false, 2, SH>)               \
+               : (f64 ? k_oras_2w<true, 0, SH> : k_oras_2w<false, 0, SH>))
+        fn = shared_per_seam(o) > 0 ? DI_ORAS_SEL(true) : DI_ORAS_SEL(false);
+#undef DI_ORAS_SEL
+        kern = (const void*)fn;
         oc = cached_occupancy(kern, 64, smem, Smem2W::bytes(true, pm != 0), &nsm);
     } else {
         smem = ((size_t)Tile2W::FIXED + (rhs_zero ? 0 : (size_t)2 * B * B)) * sizeof(float);
@@ -3172,26 +3100,14 @@ cudaError_t launch_oras_2w(const float* u_in, int zero_in, const float* rhs, int
     if (grid < 1) grid = 1;
     if (ev) record_event(ev[0], s);
     if (precision == 0) {
-#define DI_ORAS_F(F, PR)                                                                         \
-    k_oras_2w<F, PR><<<grid, 64, smem, s>>>(u_in, zero_in, rhs, rhs_zero, mbits, wpr, w, h, C, o, \
-                                            nbx, nby, alpha, iters, rtol2, u_out, planes, maxupd, \
-                                            chan_inner, tm_u, tm_b, use_tma, errflag, step_count, \
-                                            pro_e, wH, hH, pro_max, tm_e, use_tma_e)
-        if (pm == 1) {
-            if (f64) DI_ORAS_F(true, 1);
-            else DI_ORAS_F(false, 1);
-        } else if (pm == 2) {
-            if (f64) DI_ORAS_F(true, 2);
-            else DI_ORAS_F(false, 2);
-        } else {
-            if (f64) DI_ORAS_F(true, 0);
-            else DI_ORAS_F(false, 0);
-        }
-#undef DI_ORAS_F
+        fn<<<grid, 64, smem, s>>>(u_in, zero_in, rhs, rhs_zero, mbits, wpr, w, h, C, o, nbx, nby,
+                                  alpha, iters, rtol2, u_out, parked, maxupd, chan_inner, tm_u,
+                                  tm_b, use_tma, errflag, step_count, pro_e, wH, hH, pro_max,
+                                  tm_e, use_tma_e);
     } else {
 #define DI_ORAS_H(H, TU, F)                                                                     \
     run_oras_2w_h<H, TU, F>(grid, smem, s, u_in, zero_in, rhs, rhs_zero, mbits, wpr, w, h, C, o, \
-                            nbx, nby, alpha, iters, rtol2, u_out, planes, maxupd, chan_inner,   \
+                            nbx, nby, alpha, iters, rtol2, u_out, parked, maxupd, chan_inner,   \
                             step_count)
         if (precision == 1) {
             if (stor != kF32) DI_ORAS_H(HalfT, __half, false);
@@ -3208,13 +3124,13 @@ cudaError_t launch_oras_2w(const float* u_in, int zero_in, const float* rhs, int
     if (ev) record_event(ev[1], s);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    return launch_combine(planes, w, h, C, B, o, nbx, nby, u_out, s, stor);
+    return launch_combine<B>(parked, w, h, C, o, nbx, nby, u_out, s, stor);
 }
 
 template <int B>
 cudaError_t launch_oras_t(const float* u_in, int zero_in, const float* rhs, int rhs_zero,
                           const uint32_t* mbits, int wpr, int w, int h, int C, int o, float alpha,
-                          int iters, float rtol2, float* u_out, float* planes, unsigned* maxupd,
+                          int iters, float rtol2, float* u_out, float* parked, unsigned* maxupd,
                           cudaStream_t s, cudaEvent_t* ev,
                           unsigned long long* step_count) {
     const int nbx = axis_blocks(w, B, o), nby = axis_blocks(h, B, o);
@@ -3233,50 +3149,31 @@ cudaError_t launch_oras_t(const float* u_in, int zero_in, const float* rhs, int 
     if (grid < 1) grid = 1;
     if (ev) record_event(ev[0], s);
     k_oras_warp<B><<<grid, 32, smem, s>>>(u_in, zero_in, rhs, rhs_zero, mbits, wpr, w, h, C, o,
-                                          nbx, nby, alpha, iters, rtol2, u_out, planes, maxupd,
+                                          nbx, nby, alpha, iters, rtol2, u_out, parked, maxupd,
                                           chan_inner, step_count);
     count();
     if (ev) record_event(ev[1], s);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    return launch_combine(planes, w, h, C, B, o, nbx, nby, u_out, s, kF32);
+    return launch_combine<B>(parked, w, h, C, o, nbx, nby, u_out, s, kF32);
 }
 
-template <class TU>
-cudaError_t launch_combine_t(float* planes, int w, int h, int C, int B, int o, int nbx, int nby,
-                             TU* u_out, cudaStream_t s) {
-    cudaError_t e = cudaSuccess;
-    // Overlap 2 gives 0/1 weights: no pixel is shared, the combine is empty.
-    const int nsh = shared_per_seam(o);
-    const int sb = B - o;
-    const float inv_s = 1.f / (float)sb;
-    if (nsh > 0 && nby > 1) {
-        dim3 grid_r((unsigned)((w + 255) / 256), (unsigned)((nby - 1) * nsh), (unsigned)C);
-        k_combine_rows<TU><<<grid_r, 256, 0, s>>>(planes, w, h, sb, o, nbx, nby, inv_s, u_out);
-        count();
-        e = cudaGetLastError();
-        if (e != cudaSuccess) return e;
-    }
-    const int nseams = nbx - 1;
-    if (nsh > 0 && nbx > 1 && nseams > 0) {
-        const int rows = 256 / nsh > 0 ? 256 / nsh : 1;
-        dim3 blk_c((unsigned)nsh, (unsigned)rows);
-        dim3 grid_c((unsigned)((h + rows - 1) / rows), (unsigned)nseams, (unsigned)C);
-        k_combine_cols<TU><<<grid_c, blk_c, 0, s>>>(planes, w, h, sb, o, nbx, nby, inv_s, u_out);
-        count();
-        e = cudaGetLastError();
-    }
-    return e;
-}
-
-cudaError_t launch_combine(float* planes, int w, int h, int C, int B, int o, int nbx, int nby,
+template <int B>
+cudaError_t launch_combine(const float* parked, int w, int h, int C, int o, int nbx, int nby,
                            float* u_out, cudaStream_t s, int stor) {
+    // Overlap 2 gives 0/1 weights: no pixel is shared, nothing to add.
+    if (shared_per_seam(o) == 0 || nbx * nby == 1) return cudaSuccess;
+    const dim3 grid((unsigned)((nbx * C + 7) / 8), (unsigned)nby, 3);
     if (stor == kF16)
-        return launch_combine_t(planes, w, h, C, B, o, nbx, nby, reinterpret_cast<__half*>(u_out), s);
-    if (stor == kBF16)
-        return launch_combine_t(planes, w, h, C, B, o, nbx, nby,
-                                reinterpret_cast<__nv_bfloat16*>(u_out), s);
-    return launch_combine_t(planes, w, h, C, B, o, nbx, nby, u_out, s);
+        k_combine<__half, B><<<grid, 256, 0, s>>>(parked, w, h, C, o, nbx, nby,
+                                                  reinterpret_cast<__half*>(u_out));
+    else if (stor == kBF16)
+        k_combine<__nv_bfloat16, B><<<grid, 256, 0, s>>>(parked, w, h, C, o, nbx, nby,
+                                                         reinterpret_cast<__nv_bfloat16*>(u_out));
+    else
+        k_combine<float, B><<<grid, 256, 0, s>>>(parked, w, h, C, o, nbx, nby, u_out);
+    count();
+    return cudaGetLastError();
 }
 
 }  // namespace
@@ -3613,7 +3510,7 @@ cudaError_t launch_pack_mask(const uint8_t* c, int w, int h, uint32_t* bits,
 
 cudaError_t launch_oras(const float* u_in, int zero_in, const float* rhs, int rhs_zero,
                         const uint32_t* mbits, int w, int h, int C, int B, int o, float alpha,
-                        int iters, float rtol2, float* u_out, float* planes, unsigned* maxupd,
+                        int iters, float rtol2, float* u_out, float* parked, unsigned* maxupd,
                         cudaStream_t s, cudaEvent_t* ev, int precision, unsigned* errflag,
                         unsigned long long* step_count, int stor, bool f64, const float* pro_e,
                         unsigned* pro_max, int pro_mode) {
@@ -3622,14 +3519,14 @@ cudaError_t launch_oras(const float* u_in, int zero_in, const float* rhs, int rh
     switch (B) {
         case 32:
             return launch_oras_2w(u_in, zero_in, rhs, rhs_zero, mbits, wpr, w, h, C, o, alpha,
-                                  iters, rtol2, u_out, planes, maxupd, s, ev, precision, errflag,
+                                  iters, rtol2, u_out, parked, maxupd, s, ev, precision, errflag,
                                   step_count, stor, f64, pro_e, pro_max, pro_mode);
         case 16:
             return launch_oras_t<16>(u_in, zero_in, rhs, rhs_zero, mbits, wpr, w, h, C, o, alpha,
-                                     iters, rtol2, u_out, planes, maxupd, s, ev, step_count);
+                                     iters, rtol2, u_out, parked, maxupd, s, ev, step_count);
         case 8:
             return launch_oras_t<8>(u_in, zero_in, rhs, rhs_zero, mbits, wpr, w, h, C, o, alpha,
-                                    iters, rtol2, u_out, planes, maxupd, s, ev, step_count);
+                                    iters, rtol2, u_out, parked, maxupd, s, ev, step_count);
         default:
             return cudaErrorInvalidValue;
     }
