@@ -850,6 +850,12 @@ __device__ __forceinline__ float res_stencil(float b, float deg, float c, float 
     return b - (deg * c - (up + dn + l + r));
 }
 
+// The same in FP64 from the negated degree nd.
+__device__ __forceinline__ float res_f64(float b, float nd, float c, float up, float dn, float l,
+                                         float r) {
+    return res_stencil<true>(b, -nd, c, up, dn, l, r);
+}
+
 // Partition-of-unity weight of block k (of nb along an axis, stride s,
 // overlap o) at local coordinate l (Section 3.1): 0 at the block's outermost
 // overlap pixel, 1 at its innermost one, linear in between (1/2 for o = 1).
@@ -1248,14 +1254,16 @@ k_oras_warp(const float* __restrict__ u_in, int zero_in, const float* __restrict
     }
 }
 
-// One ORAS iteration for 32x32 blocks with two warps per block (one per half
-// of the rows), so every lane keeps 8 packed pairs per CG vector instead of
-// 16 and twice as many warps fit on an SM.  Warp wi owns rows 16wi .. 16wi+15
-// of every column; pair k of a lane = rows (16wi + k, 16wi + k + 8).  The row
-// pair at the seam (15 | 16) is exchanged through shared memory: each warp
-// publishes its seam row of r with the r.r partial sum, and rebuilds the
-// partner's seam row of p = r + beta p from it.  Two 64-thread barriers per CG
-// step (p.Ap and r.r).  Everything else as in k_oras_warp.
+// One ORAS iteration for 32x32 blocks with two warps per block (warp wi owns
+// rows 16wi .. 16wi+15), 16 pixels per thread.  Everything but the layout as in
+// k_oras_warp.
+//
+// k_oras_2w_h (16-bit iterates): lane = block column; pair k of a lane = rows
+// (16wi + k, 16wi + k + 8).  The FP32 kernels (k_oras_2w, k_batch_oras): see
+// BlockThread.  The row pair at the seam (15 | 16) is exchanged through shared
+// memory: each warp publishes its seam row of r with the r.r partial sum, and
+// rebuilds the partner's seam row of p = r + beta p from it.  Two 64-thread
+// barriers per CG step (p.Ap and r.r).
 struct Tile2W {
     static constexpr int B = 32, TH = 34, P = 34, TILE = TH * P;
     // shared floats: two halo tiles, row weights, two rhs tiles (optional)
@@ -1287,59 +1295,425 @@ struct Smem2W {
     }
 };
 
-// The start of an iteration formed by prolongation inside a 32x32 block's
-// tile (Section 4.4's cell-centred weights): the block pixels of this
-// thread's column (x0 and y0 + row0 are even, so row row0 + k has parent
-// patch row 1 + row0 / 2 + k / 2 and takes the coarse row above it for even
-// k, below it for odd k; the column likewise), then the halo pixels the
-// residual reads: warp 0 the row above the block and the column left of it,
-// warp 1 the row below and the column right of it, one pixel of each per
-// lane (block pixels of a neighbouring block, which counts them in the
-// maximum).  pe: the block's coarse patch (cell (r, q) = coarse row
-// y0 / 2 - 1 + r, column x0 / 2 - 1 + q, pitch Smem2W::EPW, clamped to the
-// level); mbk: the known bits of the thread's block pixels, hk: of its two
-// halo pixels (known or off the image).  ADD: u + P e at unknown pixels
-// (a correction), else P e there (an interpolated solution); known pixels
-// keep their tile value.  pmax gains the largest |P e| over the unknown
-// block pixels.  Branch-free (every patch index stays inside the patch); the
-// ten patch rows of both columns and the sixteen tile values are read before
-// anything is stored (the stores could alias them otherwise), so the loads
-// are in flight together.
+// ---- the local problem of a 32x32 block, FP32 (k_oras_2w, k_batch_oras) ------
+//
+// A thread owns two adjacent columns of eight rows: lane = 16 g + l, columns
+// cl = 2l and 2l + 1, and the rows of lane group g of warp wi counted from r0
+// in direction dr, so that local row 7 of the two groups of a warp are
+// neighbours and local row 0 is the block's outer row (g = 0: rows 0.. and
+// 31..) or the row at the warp seam (g = 1: rows 15.. and 16..).  A CG vector
+// is eight packed pairs, pair 4c + k = local rows (k, k + 4) of column cl + c.
+// Then half of the horizontal neighbours are the thread's own pairs (the other
+// half one 64-bit shuffle within 16 lanes each), local row 8 is one 32-bit
+// shuffle per column, local row -1 is the partner warp's seam row (kept as
+// pb, zero for g = 0) and no select on the row group is left in the stencil: 28
+// lane shuffles per warp and CG step, where the lane = column layout took 42
+// and where shuffles and shared-memory accesses share one pipe.  Tile loads and
+// the write of u are 8-byte words.  4K RGB, overlap 2: 13.6 us per CG step and
+// 202 us for ten (lane = column layout: 16.0 and 229), 178 warp instructions per
+// warp and step (221); with the correction's prolongation 240 us (257).
+struct BlockThread {
+    int lane, wi, g, l;
+    int cl;      // first of the two columns
+    int r0, dr;  // block row of local row 0, direction
+    __device__ __forceinline__ explicit BlockThread(int t) {
+        lane = t & 31;
+        wi = t >> 5;
+        g = lane >> 4;
+        l = lane & 15;
+        cl = 2 * l;
+        r0 = wi ? (g ? 16 : 31) : (g ? 15 : 0);
+        dr = wi == g ? 1 : -1;
+    }
+};
+
+// A_i on a thread's 16 pixels: -(diagonal) and the keep factors (0 on known
+// pixels and off the image).  Blocks of full height have one diagonal per
+// column but for local row 0, so d and e hold it; in blocks clipped by the
+// image's lower edge d holds the horizontal part and s_nv the vertical one.
+struct BlockOp {
+    f2 d[2], e[2];   // per column: the pairs 1..3, pair 0
+    f2 keep[8];
+    f2 ml, mr;       // 0/1: the left / right neighbour column is in the block
+    f2 nd;           // -(degree of A) of the two columns where both vertical neighbours exist
+    bool full;       // full height
+};
+
+// rowm: in lane i < 16 the mask bits of block row 16 wi + i (columns x0 ..
+// x0 + 31).
+__device__ __forceinline__ void block_operator(BlockOp& op, const BlockThread& bt, uint32_t rowm,
+                                               int x0, int y0, int bw, int bh, int w, int h,
+                                               float alpha) {
+    constexpr int B = 32;
+    uint32_t kn = 0;
+    const int src = bt.r0 - 16 * bt.wi;
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+        const uint32_t v = __shfl_sync(kFull, rowm, src + bt.dr * j) >> bt.cl;
+        kn |= ((v & 1u) << j) | ((v & 2u) << (7 + j));
+    }
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        const int b = 8 * (i >> 2) + (i & 3);
+        op.keep[i] = pk(((kn >> b) & 1u) ? 0.f : 1.f, ((kn >> (b + 4)) & 1u) ? 0.f : 1.f);
+    }
+    const float ml = bt.l > 0 ? 1.f : 0.f, mr = bt.l < 15 ? 1.f : 0.f;
+    op.ml = pk(ml, ml);
+    op.mr = pk(mr, mr);
+    op.full = bh == B;
+    // vertical coupling of local row 0 in a block of full height
+    const float v0 = bt.g ? 2.f
+                          : 1.f + ((bt.wi == 0 ? y0 > 0 : y0 + B < h) ? alpha : 0.f);
+    float dh[2];
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+        const int col = bt.cl + c, gx = x0 + col;
+        dh[c] = (float)((gx > 0) + (gx < w - 1));
+        const float hc = (col > 0 ? 1.f : (gx > 0 ? alpha : 0.f)) +
+                         (col + 1 < bw ? 1.f : (gx < w - 1 ? alpha : 0.f));
+        const float d = op.full ? -(hc + 2.f) : -hc;
+        op.d[c] = pk(d, d);
+        op.e[c] = pk(-(hc + v0), d);
+    }
+    op.nd = pk(-(dh[0] + 2.f), -(dh[1] + 2.f));
+}
+// The vertical part of a clipped block's diagonal into s_nv (16 pairs), read in
+// block_cg after its first barrier; called after the barrier that ends the
+// previous task's reads.
+__device__ __forceinline__ void clipped_diagonal(const BlockThread& bt, int y0, int bh, int h,
+                                                 float alpha, f2* s_nv) {
+    if (bt.l >= 4) return;
+    float vc[2];
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+        const int ly = bt.r0 + bt.dr * (bt.l + 4 * e), gy = y0 + ly;
+        vc[e] = (ly > 0 ? 1.f : (gy > 0 ? alpha : 0.f)) +
+                (ly + 1 < bh ? 1.f : (gy < h - 1 ? alpha : 0.f));
+    }
+    s_nv[(2 * bt.wi + bt.g) * 4 + bt.l] = pk(-vc[0], -vc[1]);
+}
+
+// Two adjacent words of a tile; EVEN: at an 8-byte boundary.
+template <bool EVEN>
+__device__ __forceinline__ f2 ld_pair(const float* p) {
+    if (EVEN) return *reinterpret_cast<const f2*>(p);
+    return pk(p[0], p[1]);
+}
+
+// r = b - A u on the block (0 on known pixels).  tc: the tile's word of local
+// row 0, column cl (pitch folded into ts = dr * pitch); bc, bs: the same of the
+// right-hand side tile (RHS0: 0 off the mask); INT: no row of the block on the
+// image's top or bottom row, so every vertical degree is 2.  A thread walks its
+// columns, so a row's centre is the next row's neighbour; the two columns of a
+// row are a packed pair until the masked result goes to its CG pairs.
+template <bool F64, bool RHS0, bool INT, bool EVEN>
+__device__ __forceinline__ void block_residual(f2 (&r)[8], const BlockOp& op,
+                                               const BlockThread& bt, const float* tc, int ts,
+                                               const float* bc, int bs, int zero_in, int y0,
+                                               int h) {
+    f2 rv[8];
+    f2 up = 0ull, cen = 0ull;
+    if (!zero_in) {
+        up = ld_pair<EVEN>(tc - ts);
+        cen = ld_pair<EVEN>(tc);
+    }
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+        f2 v = 0ull;
+        if (!RHS0) {
+            v = ld_pair<EVEN>(bc);
+            bc += bs;
+        }
+        if (!zero_in) {
+            const float l = tc[-1], rt = tc[2];
+            tc += ts;
+            const f2 dn = ld_pair<EVEN>(tc);
+            f2 nd = op.nd;
+            if (!INT) {
+                const int gy = y0 + bt.r0 + bt.dr * j;
+                const float e = (float)((gy == 0) + (gy == h - 1));
+                nd = add2(nd, pk(e, e));
+            }
+            if (F64) {
+                const float b0 = lo2(v), b1 = hi2(v);
+                v = pk(res_f64(b0, lo2(nd), lo2(cen), lo2(up), lo2(dn), l, hi2(cen)),
+                       res_f64(b1, hi2(nd), hi2(cen), hi2(up), hi2(dn), lo2(cen), rt));
+            } else {
+                const f2 nb = add2(add2(up, dn), pk(l + hi2(cen), lo2(cen) + rt));
+                const f2 t = fma2(nd, cen, nb);  // -(A u)
+                v = RHS0 ? t : add2(v, t);
+            }
+            up = cen;
+            cen = dn;
+        }
+        rv[j] = v;
+    }
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        r[k] = pk(lo2(rv[k]) * lo2(op.keep[k]), lo2(rv[k + 4]) * hi2(op.keep[k]));
+        r[4 + k] = pk(hi2(rv[k]) * lo2(op.keep[4 + k]), hi2(rv[k + 4]) * hi2(op.keep[4 + k]));
+    }
+}
+
+// Shared words of block_cg.
+struct BlockShared {
+    float red1[2], red2[2];
+    float2 seam[2][16];
+    f2 nv[16];
+};
+
+// a / b for normal b > 0: one approximate reciprocal (both warps of a block
+// compute it from the same words, so they agree).
+__device__ __forceinline__ float quotient(float a, float b) {
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(b));
+    return a * r;
+}
+
+// Up to `iters` CG steps on A_i x = r from x = 0 (r is overwritten); both
+// warps of the block.  rtol2 >= 0: relative stop (r.r <= max(rtol2, 1e-14)
+// (r.r)_0); rtol2 < 0: also stop once r.r <= -rtol2 (an absolute level, or the
+// FP32 floor).  The last step updates x alone.  Returns the completed steps.
+// Bound by the register file: an instruction takes half a cycle per 32-bit
+// operand word it reads (a packed FMA of three distinct pairs 3 cycles, an
+// add 2, a scalar add 1), which is why nothing here trades fewer
+// instructions for more operands, and more warps per SM do not help.
+template <bool FULL>
+__device__ __forceinline__ unsigned block_cg_t(f2 (&x)[8], f2 (&r)[8], const BlockOp& op,
+                                               const BlockThread& bt, int iters, float rtol2,
+                                               BlockShared& sh) {
+    f2 p[8], q[8];
+    f2 acc0, acc1;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        p[i] = r[i];
+        x[i] = 0ull;
+        if (i == 0) acc0 = mul2(r[i], r[i]);
+        else if (i == 4) acc1 = mul2(r[i], r[i]);
+        else if (i < 4) acc0 = fma2(r[i], r[i], acc0);
+        else acc1 = fma2(r[i], r[i], acc1);
+    }
+    acc0 = add2(acc0, acc1);
+    if (bt.g) sh.seam[bt.wi][bt.l] = make_float2(lo2(r[0]), lo2(r[4]));
+    float part = warp_sum(lo2(acc0) + hi2(acc0));
+    if (bt.lane == 0) sh.red2[bt.wi] = part;
+    __syncthreads();
+    float rr = sh.red2[0] + sh.red2[1];
+    float2 pb = make_float2(0.f, 0.f);  // local row -1 of p
+    if (bt.g) pb = sh.seam[bt.wi ^ 1][bt.l];
+    // never below the smallest normal, so that the quotients stay finite
+    const float rr_stop = fmaxf(rtol2 >= 0.f ? fmaxf(rtol2, 1e-14f) * rr : fmaxf(1e-14f * rr, -rtol2),
+                                FLT_MIN);
+    const f2* nv = sh.nv + (2 * bt.wi + bt.g) * 4;
+    int it = 0;
+    while (it < iters && rr > rr_stop) {  // rr is identical in both warps
+        const float dn0 = __shfl_xor_sync(kFull, hi2(p[3]), 16);  // local row 8
+        const float dn1 = __shfl_xor_sync(kFull, hi2(p[7]), 16);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const f2 left = __shfl_up_sync(kFull, p[4 + k], 1, 16);
+            const f2 right = __shfl_down_sync(kFull, p[k], 1, 16);
+            // vertical neighbours: local row -1 is the partner's, local row 8 the
+            // other row group's (their pairs as two scalar sums: packing the
+            // halves first takes more instructions)
+            f2 n0, n1;
+            if (k == 0) {
+                n0 = pk(pb.x + lo2(p[1]), lo2(p[3]) + hi2(p[1]));
+                n1 = pk(pb.y + lo2(p[5]), lo2(p[7]) + hi2(p[5]));
+            } else if (k == 3) {
+                n0 = pk(lo2(p[2]) + hi2(p[0]), hi2(p[2]) + dn0);
+                n1 = pk(lo2(p[6]) + hi2(p[4]), hi2(p[6]) + dn1);
+            } else {
+                n0 = add2(p[k - 1], p[k + 1]);
+                n1 = add2(p[3 + k], p[5 + k]);
+            }
+            n0 = add2(n0, p[4 + k]);
+            n1 = add2(n1, p[k]);
+            n0 = fma2(op.ml, left, n0);
+            n1 = fma2(op.mr, right, n1);
+            f2 g0, g1;
+            if (FULL) {
+                g0 = k ? op.d[0] : op.e[0];
+                g1 = k ? op.d[1] : op.e[1];
+            } else {
+                const f2 v = nv[k];
+                g0 = add2(v, op.d[0]);
+                g1 = add2(v, op.d[1]);
+            }
+            // -(A_i p), 0 on the mask
+            q[k] = mul2(fma2(g0, p[k], n0), op.keep[k]);
+            q[4 + k] = mul2(fma2(g1, p[4 + k], n1), op.keep[4 + k]);
+            acc0 = k ? fma2(p[k], q[k], acc0) : mul2(p[k], q[k]);
+            acc1 = k ? fma2(p[4 + k], q[4 + k], acc1) : mul2(p[4 + k], q[4 + k]);
+        }
+        acc0 = add2(acc0, acc1);
+        part = warp_sum(lo2(acc0) + hi2(acc0));
+        if (bt.lane == 0) sh.red1[bt.wi] = part;
+        __syncthreads();
+        const float pq = -(sh.red1[0] + sh.red1[1]);
+        if (!(pq >= FLT_MIN && pq <= FLT_MAX)) break;
+        const float a = quotient(rr, pq);
+        const f2 a2 = pk(a, a);
+        if (++it == iters) {
+#pragma unroll
+            for (int i = 0; i < 8; ++i) x[i] = fma2(a2, p[i], x[i]);
+            break;
+        }
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            x[i] = fma2(a2, p[i], x[i]);
+            r[i] = fma2(a2, q[i], r[i]);
+            if (i == 0) acc0 = mul2(r[i], r[i]);
+            else if (i == 4) acc1 = mul2(r[i], r[i]);
+            else if (i < 4) acc0 = fma2(r[i], r[i], acc0);
+            else acc1 = fma2(r[i], r[i], acc1);
+        }
+        acc0 = add2(acc0, acc1);
+        if (bt.g) sh.seam[bt.wi][bt.l] = make_float2(lo2(r[0]), lo2(r[4]));
+        part = warp_sum(lo2(acc0) + hi2(acc0));
+        if (bt.lane == 0) sh.red2[bt.wi] = part;
+        __syncthreads();
+        const float rrn = sh.red2[0] + sh.red2[1];
+        const float beta = quotient(rrn, rr);
+        rr = rrn;
+        const f2 b2 = pk(beta, beta);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) p[i] = fma2(b2, p[i], r[i]);
+        if (bt.g) {
+            const float2 sv = sh.seam[bt.wi ^ 1][bt.l];
+            pb.x = fmaf(beta, pb.x, sv.x);
+            pb.y = fmaf(beta, pb.y, sv.y);
+        }
+    }
+    return (unsigned)it;
+}
+__device__ __forceinline__ unsigned block_cg(f2 (&x)[8], f2 (&r)[8], const BlockOp& op,
+                                             const BlockThread& bt, int iters, float rtol2,
+                                             BlockShared& sh) {
+    return op.full ? block_cg_t<true>(x, r, op, bt, iters, rtol2, sh)
+                   : block_cg_t<false>(x, r, op, bt, iters, rtol2, sh);
+}
+
+// Overlap 2: bit j of the local rows whose weight is 1 (all but a block edge
+// inside the image) and that lie in the image.
+__device__ __forceinline__ uint32_t own_rows(const BlockThread& bt, int ky, int nby, int bh) {
+    uint32_t m = bt.g || (bt.wi == 0 ? ky == 0 : ky == nby - 1) ? 0xffu : 0xfeu;
+#pragma unroll
+    for (int j = 0; j < 8; ++j)
+        if (bt.r0 + bt.dr * j >= bh) m &= ~(1u << j);
+    return m;
+}
+
+// Local row j of column c of a solution.
+__device__ __forceinline__ float block_value(const f2 (&x)[8], int c, int j) {
+    return j < 4 ? lo2(x[4 * c + j]) : hi2(x[4 * c + j - 4]);
+}
+
+// The write of 0/1 weights (overlap 2): each pixel is written by the one block
+// whose weight is 1 there, with u_in (the tile; zero_in: 0) added.  up: u_out
+// at local row 0, column cl; us: its step to the next local row; own0, own1:
+// the columns are the block's own; rows: bit j of a local row j of its own
+// (ALL: rows 1 .. 7 are); vec: up is at an 8-byte boundary in every row.  vmax
+// gains the largest |x| written.  A lane with one column of its own stores a
+// word, the others two, without a branch on it.
+template <bool ALL>
+__device__ __forceinline__ void block_write01(const f2 (&x)[8], const float* tc, int ts,
+                                              int zero_in, float* up, ptrdiff_t us, bool own0,
+                                              bool own1, uint32_t rows, bool vec, float& vmax) {
+    const bool two = own0 && own1, one = own0 != own1;
+    float m0 = 0.f, m1 = 0.f;
+    const int oc = own0 ? 0 : 1;
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+        const bool ok = (ALL && j > 0) || ((rows >> j) & 1u);
+        const float v0 = block_value(x, 0, j), v1 = block_value(x, 1, j);
+        f2 u = 0ull;
+        if (!zero_in) u = ld_pair<true>(tc);
+        const float a = lo2(u) + v0, b = hi2(u) + v1;
+        if (vec) {
+            if (ok && two) *reinterpret_cast<f2*>(up) = pk(a, b);
+            if (ok && one) up[oc] = own0 ? a : b;
+        } else {
+            if (ok && own0) up[0] = a;
+            if (ok && own1) up[1] = b;
+        }
+        if (ok) {
+            m0 = fmaxf(m0, fabsf(v0));
+            m1 = fmaxf(m1, fabsf(v1));
+        }
+        tc += ts;
+        up += us;
+    }
+    if (own0) vmax = fmaxf(vmax, m0);
+    if (own1) vmax = fmaxf(vmax, m1);
+}
+
+// The start of an iteration formed by prolongation inside a block's tile
+// (Section 4.4's cell-centred weights): the thread's 16 pixels (x0 and y0 are
+// even: columns cl and cl + 1 have the same parent, and local rows 2m, 2m + 1
+// too; the even local row takes the coarse row before it in the thread's
+// direction, the odd one the row after it), then the halo pixels the residual
+// reads: warp 0 the row above the block and the column left of it, warp 1 the
+// row below and the column right of it, one pixel of each per lane (block
+// pixels of a neighbouring block, which counts them in the maximum).  pe: the
+// block's coarse patch (cell (r, q) = coarse row y0 / 2 - 1 + r, column x0 / 2
+// - 1 + q, pitch Smem2W::EPW, clamped to the level); hk: bits of the thread's
+// two halo pixels (known or off the image).  ADD:
+// u + P e at unknown pixels (a correction), else P e there (an interpolated
+// solution); known pixels keep their tile value.  tw: the tile's word of the
+// halo corner.  pmax gains the largest |P e| over the unknown block pixels.
+// Branch-free (every patch index stays inside the patch); the patch rows and
+// the tile values are read before anything is stored (the stores could alias
+// them otherwise), so the loads are in flight together.
 template <bool ADD>
-__device__ __forceinline__ void prolong_into_tile(float* tw, const float* pe, int row0, int col,
-                                                  int lane, int wi, int x0, int y0, uint32_t mbk,
+__device__ __forceinline__ void prolong_into_tile(float* tw, const float* pe,
+                                                  const BlockThread& bt, const BlockOp& op,
                                                   uint32_t hk, float& pmax) {
     constexpr int EW = Smem2W::EPW, P = Smem2W::PU, B = 32;
     {
-        const int q = 1 + (col >> 1), qn = (col & 1) ? q + 1 : q - 1;
-        const float* pr = pe + (row0 >> 1) * EW;  // patch row of coarse row Yb - 1
-        float* tc = tw + (row0 + 1) * P + col + 1;
-        float ec[10], es[10], tv[16];
+        const int q = 1 + bt.l, es = bt.dr * EW, ts = bt.dr * P;
+        const float* pr = pe + (1 + (bt.r0 >> 1)) * EW + q - es;  // row before the first parent
+        float* tc = tw + (bt.r0 + 1) * P + bt.cl + 1;
+        float el[6], ec[6], er[6];
+        f2 tv[8];
 #pragma unroll
-        for (int j = 0; j < 10; ++j) {
-            ec[j] = pr[j * EW + q];
-            es[j] = pr[j * EW + qn];
+        for (int i = 0; i < 6; ++i) {
+            el[i] = pr[-1];
+            ec[i] = pr[0];
+            er[i] = pr[1];
+            pr += es;
         }
 #pragma unroll
-        for (int k = 0; k < 16; ++k) tv[k] = tc[k * P];
+        for (int j = 0; j < 8; ++j) tv[j] = ld_pair<true>(tc + j * ts);
 #pragma unroll
-        for (int k = 0; k < 16; ++k) {
-            const int jc = (k >> 1) + 1, jn = (k & 1) ? jc + 1 : jc - 1;
-            const float a = prolong_blend(ec[jc], ec[jn], es[jc], es[jn]);
-            const bool kn = (mbk >> k) & 1u;
-            tc[k * P] = kn ? tv[k] : (ADD ? __fadd_rn(tv[k], a) : a);
-            pmax = fmaxf(pmax, kn ? 0.f : fabsf(a));
+        for (int j = 0; j < 8; ++j) {
+            const int i = 1 + (j >> 1), n = (j & 1) ? i + 1 : i - 1;
+            // unknown: the keep factor of the pixel is not 0
+            const f2 kp0 = op.keep[j & 3], kp1 = op.keep[4 + (j & 3)];
+            const bool u0 = (j < 4 ? lo2(kp0) : hi2(kp0)) != 0.f;
+            const bool u1 = (j < 4 ? lo2(kp1) : hi2(kp1)) != 0.f;
+            const float b0 = prolong_blend(ec[i], ec[n], el[i], el[n]);
+            const float b1 = prolong_blend(ec[i], ec[n], er[i], er[n]);
+            const float a0 = u0 ? b0 : 0.f, a1 = u1 ? b1 : 0.f;
+            const float t0 = lo2(tv[j]), t1 = hi2(tv[j]);
+            *reinterpret_cast<f2*>(tc + j * ts) =
+                ADD ? pk(__fadd_rn(t0, a0), __fadd_rn(t1, a1)) : pk(u0 ? a0 : t0, u1 ? a1 : t1);
+            pmax = fmaxf(pmax, fmaxf(fabsf(a0), fabsf(a1)));
         }
     }
+    // x0 and y0 are even, so the parent cell of a halo pixel and the side of
+    // its neighbours depend on the thread alone
+    const int odd = bt.lane & 1, half = 1 + (bt.lane >> 1), far = bt.wi ? B / 2 + 1 : 0;
 #pragma unroll
     for (int side = 0; side < 2; ++side) {
-        const int hy = side == 0 ? (wi == 0 ? y0 - 1 : y0 + B) : y0 + lane;
-        const int hx = side == 0 ? x0 + lane : (wi == 0 ? x0 - 1 : x0 + B);
-        const int r = (hy >> 1) - (y0 >> 1) + 1, q = (hx >> 1) - (x0 >> 1) + 1;
-        const int rn = (hy & 1) ? r + 1 : r - 1, qn = (hx & 1) ? q + 1 : q - 1;
-        const float a = prolong_blend(pe[r * EW + q], pe[rn * EW + q], pe[r * EW + qn],
-                                      pe[rn * EW + qn]);
-        float* tp = tw + (hy - y0 + 1) * P + (hx - x0 + 1);
+        const float* pp = pe + (side == 0 ? far * EW + half : half * EW + far);
+        // to the neighbour across the block's edge and along it
+        const int in = (side == 0 ? EW : 1) * (bt.wi ? -1 : 1);
+        const int al = (side == 0 ? 1 : EW) * (odd ? 1 : -1);
+        const int vn = side == 0 ? in : al, hn = side == 0 ? al : in;
+        const float a = prolong_blend(pp[0], pp[vn], pp[hn], pp[vn + hn]);
+        float* tp = tw + (side == 0 ? (bt.wi ? (B + 1) * P : 0) + bt.lane + 1
+                                    : (bt.lane + 1) * P + (bt.wi ? B + 1 : 0));
         const bool kn = (hk >> side) & 1u;  // known or off the image
         const float old = *tp;
         *tp = kn ? old : (ADD ? __fadd_rn(old, a) : a);
@@ -1436,10 +1810,11 @@ __device__ __forceinline__ void tma_load_3d(unsigned dst, const CUtensorMap* map
 // the known pixels and P eH at the unknown ones (prolong_body's mode 0 with
 // u_in as b: the cascade's interpolation of the coarser level's solution).
 // Each block forms the start in its tile (block pixels and halo) before the
-// residual.  SHARED: blocks share pixels (overlap 1 or >= 3); otherwise
-// (overlap 2) the partition weights are 0 and 1.  Needs u_in (not zero_in) and an even block stride, so that the
+// residual.  OV: 0 overlap 2 (partition weights 0 and 1); blocks share pixels
+// (overlap 1 or >= 3) and 1 the block stride 32 - o is even, 2 odd (block
+// columns at odd pixels: no 8-byte words).  Needs u_in (not zero_in) and an even block stride, so that the
 // parity of a block pixel is that of its tile index.
-template <bool F64, int PRO, bool SHARED>
+template <bool F64, int PRO, int OV>
 __global__ void __launch_bounds__(64, 8)
 k_oras_2w(const float* __restrict__ u_in, int zero_in, const float* __restrict__ rhs,
           int rhs_zero, const uint32_t* __restrict__ mbits, int wpr, int w, int h, int C, int o,
@@ -1450,7 +1825,7 @@ k_oras_2w(const float* __restrict__ u_in, int zero_in, const float* __restrict__
           unsigned long long* __restrict__ step_count, const float* __restrict__ eH, int wH,
           int hH, unsigned* __restrict__ maxpro, const __grid_constant__ CUtensorMap tm_e,
           int use_tma_e) {
-    constexpr int B = 32, NP = 8, TH = Smem2W::TH, P = Smem2W::PU, PB = Smem2W::PB;
+    constexpr int B = 32, TH = Smem2W::TH, P = Smem2W::PU, PB = Smem2W::PB;
     constexpr int TILE = Smem2W::USTRIDE;
     extern __shared__ float smem_raw[];
     float* const smem = reinterpret_cast<float*>(
@@ -1459,13 +1834,12 @@ k_oras_2w(const float* __restrict__ u_in, int zero_in, const float* __restrict__
     float* const s_wy = smem + Smem2W::WY;       // [B]
     float* const s_e = smem + Smem2W::EP;        // [2][ES] if PRO
     float* const s_b = smem + (PRO ? Smem2W::RHS_PRO : Smem2W::RHS);  // [2][BSTRIDE] if rhs_zero == 0
-    __shared__ float s_red1[2], s_red2[2], s_seam[2][32];
+    __shared__ BlockShared sh;
     __shared__ __align__(8) unsigned long long s_bar[2];
 
     const int t = threadIdx.x;
-    const int lane = t & 31, wi = t >> 5;
-    const int col = lane;
-    const int row0 = 16 * wi;
+    const BlockThread bt(t);
+    const int lane = bt.lane, wi = bt.wi;
     const int s = B - o;
     const size_t n = (size_t)w * h;
     const float inv_o1 = o > 1 ? 1.f / (float)(o - 1) : 0.f;
@@ -1489,8 +1863,13 @@ k_oras_2w(const float* __restrict__ u_in, int zero_in, const float* __restrict__
     };
     uint32_t nlo = 0xffffffffu, nhi = 0xffffffffu;
     uint32_t nhk = 3u;  // PRO: bit i = halo pixel i of this thread (next block) is known or off the image
+    int px0 = 0, py0 = 0;  // origin of the block prefetched last
     auto prefetch = [&](int blk, int ch, int bs, int have_blk) {
-        const int px0 = (blk % nbx) * s, py0 = (blk / nbx) * s;
+        if (blk != have_blk) {
+            py0 = blk / nbx;
+            px0 = (blk - py0 * nbx) * s;
+            py0 *= s;
+        }
         if constexpr (PRO != 0) {
             // the coarse cells the task's prolongation reads: rows
             // (py0 >> 1) - 1 + r and columns (px0 >> 1) - 1 + q, r, q < 18
@@ -1533,9 +1912,10 @@ k_oras_2w(const float* __restrict__ u_in, int zero_in, const float* __restrict__
             }
         } else if (!zero_in) {
             // thread t copies tile column lane of the rows ty = wi, wi + 2, ...
-            // (and column 32 + lane for lane < 2)
+            // (and column 32 + lane for lane < 2); one word in, as for TMA tiles
+            // of an odd halo column, so that block column 0 is 8-byte aligned
             const float* src = u_in + ch * n;
-            float* dst = s_u + bs * TILE;
+            float* dst = s_u + bs * TILE + 1;
             const int gxa = px0 - 1 + lane, gxb = gxa + 32;
             const bool oka = gxa >= 0 && gxa < w;
             const bool okb = lane < TH - 32 && gxb < w;
@@ -1562,7 +1942,7 @@ k_oras_2w(const float* __restrict__ u_in, int zero_in, const float* __restrict__
         }
         if (!use_tma) cp_async_commit();
         if (blk != have_blk && lane < 16) {
-            const int gy = py0 + row0 + lane;
+            const int gy = py0 + 16 * wi + lane;
             if (gy < h) {
                 const uint32_t* row = mbits + (size_t)gy * wpr + (px0 >> 5);
                 nlo = __ldg(row);
@@ -1590,16 +1970,32 @@ k_oras_2w(const float* __restrict__ u_in, int zero_in, const float* __restrict__
     unsigned phase = 0;  // bit b: parity of the next completion of s_bar[b]
     prefetch(blk, ch, 0, -1);
     int buf = 0, cur_blk = -1;
-    f2 ndg[NP], keep[NP];
-    f2 ml2 = 0ull, mr2 = 0ull;
-    float wx = 0.f, dh = 0.f;
+    BlockOp op;
+    float wx0 = 0.f, wx1 = 0.f;  // column weights
     int x0 = 0, y0 = 0, bh = 0, kx = 0, ky = 0;
-    uint32_t rows_w = 0;  // bit ly: row ly of the block is in the image with weight > 0
-    uint32_t mbk = 0;     // bit k: pixel (row0 + k, col) of the block is known or off the image
+    uint32_t rows_w = 0;  // overlap 2, bit j: local row j is in the image with weight 1
     float vmax = 0.f, pmax = 0.f;
     unsigned nsteps = 0;  // completed local CG steps of this thread's tasks
+    // 8-byte stores of u_out
+    const bool vec = OV != 2 && (w & 1) == 0 && (reinterpret_cast<uintptr_t>(u_out) & 7) == 0;
 
     for (;;) {
+        const bool new_blk = blk != cur_blk;
+        if (new_blk) {
+            // the local operator, while the tile is on its way
+            cur_blk = blk;
+            ky = blk / nbx;
+            kx = blk - ky * nbx;
+            x0 = kx * s;
+            y0 = ky * s;
+            bh = min(B, h - y0);
+            // lane < 16: the mask bits of row 16 wi + lane
+            block_operator(op, bt, __funnelshift_r(nlo, nhi, x0 & 31), x0, y0, min(B, w - x0), bh,
+                           w, h, alpha);
+            wx0 = x0 + bt.cl < w ? ramp_weight(bt.cl, kx, nbx, s, o, inv_o1) : 0.f;
+            wx1 = x0 + bt.cl + 1 < w ? ramp_weight(bt.cl + 1, kx, nbx, s, o, inv_o1) : 0.f;
+            if constexpr (OV == 0) rows_w = own_rows(bt, ky, nby, bh);
+        }
         if (use_tma) {
             const unsigned bar = (unsigned)__cvta_generic_to_shared(&s_bar[buf]);
             bool ok = mbar_wait(bar, (phase >> buf) & 1u);
@@ -1615,71 +2011,25 @@ k_oras_2w(const float* __restrict__ u_in, int zero_in, const float* __restrict__
             cp_async_wait_all();
             __syncthreads();
         }
-        const uint32_t mlo = nlo, mhi = nhi, hk = nhk;
+        const uint32_t hk = nhk;
         int nb2 = blk, nc2 = ch;
         const bool more = next_task(nb2, nc2);
         if (more) prefetch(nb2, nc2, buf ^ 1, blk);
 
-        if (blk != cur_blk) {
-            cur_blk = blk;
-            kx = blk % nbx;
-            ky = blk / nbx;
-            x0 = kx * s;
-            y0 = ky * s;
-            const int bw = min(B, w - x0);
-            bh = min(B, h - y0);
-            const uint32_t rowm = __funnelshift_r(mlo, mhi, x0 & 31);  // lane < 16: row row0+lane
-            uint32_t mb = 0;
-#pragma unroll
-            for (int rr = 0; rr < 16; ++rr) {
-                const uint32_t v = __shfl_sync(kFull, rowm, rr);
-                mb |= ((v >> col) & 1u) << rr;
-            }
-            const int gx = x0 + col;
-            const float hc = (col > 0 ? 1.f : (gx > 0 ? alpha : 0.f)) +
-                             (col + 1 < bw ? 1.f : (gx < w - 1 ? alpha : 0.f));
-            dh = (float)((gx > 0) + (gx < w - 1));
-            const float ml = col > 0 ? 1.f : 0.f, mr = col < B - 1 ? 1.f : 0.f;
-            ml2 = pk(ml, ml);
-            mr2 = pk(mr, mr);
-            if (bh == B) {
-                // full height: vertical coupling count 2 except in rows 0 and 31
-                const float d2 = -(hc + 2.f);
-                const float vt = (y0 > 0 ? alpha : 0.f) + 1.f;
-                const float vb = 1.f + (y0 + B < h ? alpha : 0.f);
-#pragma unroll
-                for (int k = 0; k < NP; ++k) ndg[k] = pk(d2, d2);
-                if (wi == 0) ndg[0] = pk(-(hc + vt), d2);
-                else ndg[NP - 1] = pk(d2, -(hc + vb));
-            } else {
-#pragma unroll
-                for (int k = 0; k < NP; ++k) {
-                    float vc[2];
-#pragma unroll
-                    for (int e = 0; e < 2; ++e) {
-                        const int ly = row0 + k + 8 * e, gy = y0 + ly;
-                        vc[e] = (ly > 0 ? 1.f : (gy > 0 ? alpha : 0.f)) +
-                                (ly + 1 < bh ? 1.f : (gy < h - 1 ? alpha : 0.f));
-                    }
-                    ndg[k] = pk(-(hc + vc[0]), -(hc + vc[1]));
-                }
-            }
-#pragma unroll
-            for (int k = 0; k < NP; ++k)
-                keep[k] = pk(((mb >> k) & 1u) ? 0.f : 1.f, ((mb >> (k + 8)) & 1u) ? 0.f : 1.f);
-            mbk = mb;
-            wx = ramp_weight(col, kx, nbx, s, o, inv_o1);
-            const float wyl = ramp_weight(lane, ky, nby, s, o, inv_o1);  // row lane
-            if (t < B) s_wy[t] = wyl;
-            // s_wy is read only after the barriers of the CG below
-            rows_w = __ballot_sync(kFull, wyl > 0.f && lane < bh);
+        if (new_blk) {
+            if (!op.full) clipped_diagonal(bt, y0, bh, h, alpha, sh.nv);
+            // read only after the barriers of the CG below
+            if (OV != 0 && t < B)
+                s_wy[t] = lane < bh ? ramp_weight(lane, ky, nby, s, o, inv_o1) : 0.f;
         }
 
         // TMA tiles start at the 4-aligned column below the halo column
-        const int du = use_tma ? ((x0 - 1) & 3) : 0;
+        const int du = use_tma ? ((x0 - 1) & 3) : 1;
         const int db = use_tma ? (x0 & 3) : 0;
-        const float* tu = s_u + buf * TILE + du;
-        const float* tb = s_b + buf * Smem2W::BSTRIDE + db;
+        // local row 0, column cl of the tiles, and the steps to the next local row
+        const float* tc = s_u + buf * TILE + du + (bt.r0 + 1) * P + bt.cl + 1;
+        const float* bc = s_b + buf * Smem2W::BSTRIDE + db + bt.r0 * PB + bt.cl;
+        const int ts = bt.dr * P, bs = bt.dr * PB;
         if constexpr (PRO != 0) {
             // the start of the iteration in the tile (prolong_into_tile)
             constexpr int EW = Smem2W::EPW;  // patch pitch
@@ -1699,169 +2049,60 @@ k_oras_2w(const float* __restrict__ u_in, int zero_in, const float* __restrict__
                 }
                 __syncthreads();  // block-uniform branch
             }
-            prolong_into_tile<PRO == 1>(tw, pw, row0, col, lane, wi, x0, y0, mbk, hk, pmax);
+            prolong_into_tile<PRO == 1>(tw, pw, bt, op, hk, pmax);
             __syncthreads();  // the residual reads the other threads' columns
         }
 
-        f2 x[NP], r[NP], p[NP], q[NP];
-        f2 acc0 = 0ull, acc1 = 0ull;
-        // r = b - A u on the block (0 on the mask).  The variants: rows off the
-        // image's top and bottom rows (vertical degree 2), and b = 0 off the mask.
-        // Each run of eight rows walks down the lane's column, so a row's centre
-        // is the next row's upper neighbour (one tile load per row for the
-        // vertical neighbours instead of three).
-        auto residual = [&](auto interior, auto rhs0) {
-            float rv[2 * NP];  // rows row0 .. row0 + 15
-#pragma unroll
-            for (int e = 0; e < 2; ++e) {
-                const float* cb = tu + (row0 + 8 * e + 1) * P + col + 1;  // centre of row 8e
-                float up = 0.f, cen = 0.f;
-                if (!zero_in) {
-                    up = cb[-P];
-                    cen = cb[0];
-                }
-#pragma unroll
-                for (int k = 0; k < NP; ++k) {
-                    const int ly = row0 + k + 8 * e, gy = y0 + ly;
-                    float v = decltype(rhs0)::value ? 0.f : tb[ly * PB + col];
-                    if (!zero_in) {
-                        const float* c0 = cb + k * P;
-                        const float dn = c0[P];
-                        const float dv = decltype(interior)::value
-                                             ? 2.f : (float)((gy > 0) + (gy < h - 1));
-                        v = res_stencil<F64>(v, dh + dv, cen, up, dn, c0[-1], c0[1]);
-                        up = cen;
-                        cen = dn;
-                    }
-                    rv[k + NP * e] = v;
-                }
-            }
-#pragma unroll
-            for (int k = 0; k < NP; ++k) {
-                r[k] = mul2(pk(rv[k], rv[k + NP]), keep[k]);
-                p[k] = r[k];
-                x[k] = 0ull;
-                if (k & 1) acc1 = fma2(r[k], r[k], acc1);
-                else acc0 = fma2(r[k], r[k], acc0);
-            }
-        };
+        f2 x[8], r[8];
+        constexpr bool EV = OV != 2;
         if (y0 > 0 && y0 + B < h) {
-            if (rhs_zero) residual(std::true_type{}, std::true_type{});
-            else residual(std::true_type{}, std::false_type{});
+            if (rhs_zero) block_residual<F64, true, true, EV>(r, op, bt, tc, ts, bc, bs, zero_in, y0, h);
+            else block_residual<F64, false, true, EV>(r, op, bt, tc, ts, bc, bs, zero_in, y0, h);
         } else {
-            if (rhs_zero) residual(std::false_type{}, std::true_type{});
-            else residual(std::false_type{}, std::false_type{});
+            if (rhs_zero) block_residual<F64, true, false, EV>(r, op, bt, tc, ts, bc, bs, zero_in, y0, h);
+            else block_residual<F64, false, false, EV>(r, op, bt, tc, ts, bc, bs, zero_in, y0, h);
         }
-        acc0 = add2(acc0, acc1);
-        // seam rows: warp 0 publishes its row 15 (hi of pair 7), warp 1 its row 16 (lo of pair 0)
-        s_seam[wi][lane] = wi == 0 ? hi2(r[NP - 1]) : lo2(r[0]);
-        float part = warp_sum(lo2(acc0) + hi2(acc0));
-        if (lane == 0) s_red2[wi] = part;
-        __syncthreads();
-        float rr = s_red2[0] + s_red2[1];
-        float pb = s_seam[wi ^ 1][lane];  // partner's seam row of p
-        // rtol2 >= 0: relative stop (r.r <= max(rtol2, 1e-14) (r.r)_0); rtol2 < 0:
-        // also stop once r.r <= -rtol2 (an absolute level, or the FP32 floor)
-        const float rr_stop = rtol2 >= 0.f ? fmaxf(rtol2, 1e-14f) * rr
-                                           : fmaxf(1e-14f * rr, -rtol2);
+        nsteps += block_cg(x, r, op, bt, iters, rtol2, sh);
 
-        for (int it = 0; it < iters; ++it) {
-            if (!(rr > rr_stop)) break;  // rr is identical in both warps
-            const f2 pu = wi == 0 ? pk(0.f, lo2(p[NP - 1])) : pk(pb, lo2(p[NP - 1]));
-            const f2 pd = wi == 0 ? pk(hi2(p[0]), pb) : pk(hi2(p[0]), 0.f);
-            acc0 = 0ull;
-            acc1 = 0ull;
-#pragma unroll
-            for (int k = 0; k < NP; ++k) {
-                const f2 left = __shfl_up_sync(kFull, p[k], 1);
-                const f2 right = __shfl_down_sync(kFull, p[k], 1);
-                const f2 up = k > 0 ? p[k - 1] : pu;
-                const f2 dn = k < NP - 1 ? p[k + 1] : pd;
-                f2 nbs = add2(up, dn);
-                nbs = fma2(ml2, left, nbs);
-                nbs = fma2(mr2, right, nbs);
-                const f2 qk = mul2(fma2(ndg[k], p[k], nbs), keep[k]);  // -(A_i p), 0 on the mask
-                q[k] = qk;
-                if (k & 1) acc1 = fma2(p[k], qk, acc1);
-                else acc0 = fma2(p[k], qk, acc0);
-            }
-            acc0 = add2(acc0, acc1);
-            part = warp_sum(lo2(acc0) + hi2(acc0));
-            if (lane == 0) s_red1[wi] = part;
-            __syncthreads();
-            const float pq = -(s_red1[0] + s_red1[1]);
-            if (!(pq > 0.f) || pq == INFINITY) break;
-            const float a = __fdividef(rr, pq);
-            const f2 a2 = pk(a, a);
-            acc0 = 0ull;
-            acc1 = 0ull;
-#pragma unroll
-            for (int k = 0; k < NP; ++k) {
-                x[k] = fma2(a2, p[k], x[k]);
-                r[k] = fma2(a2, q[k], r[k]);
-                if (k & 1) acc1 = fma2(r[k], r[k], acc1);
-                else acc0 = fma2(r[k], r[k], acc0);
-            }
-            acc0 = add2(acc0, acc1);
-            s_seam[wi][lane] = wi == 0 ? hi2(r[NP - 1]) : lo2(r[0]);
-            part = warp_sum(lo2(acc0) + hi2(acc0));
-            if (lane == 0) s_red2[wi] = part;
-            __syncthreads();
-            const float rrn = s_red2[0] + s_red2[1];
-            const float beta = __fdividef(rrn, rr);
-            rr = rrn;
-            const f2 b2 = pk(beta, beta);
-#pragma unroll
-            for (int k = 0; k < NP; ++k) p[k] = fma2(b2, p[k], r[k]);
-            pb = fmaf(beta, pb, s_seam[wi ^ 1][lane]);
-            ++nsteps;
-        }
-
-        float* uo = u_out + ch * n;
-        const bool colok = x0 + col < w;
-        if constexpr (!SHARED) {
-            // 0/1 weights (overlap 2): each pixel is written by the one block
-            // whose weight is 1 there, with u_in added
-            if (colok && wx > 0.f) {
-                float* uol = uo + (size_t)(y0 + row0) * w + x0 + col;
-                const float* tol = tu + (row0 + 1) * P + col + 1;
-#pragma unroll
-                for (int e = 0; e < 2; ++e) {
-#pragma unroll
-                    for (int k = 0; k < NP; ++k) {
-                        const int j = k + 8 * e;
-                        if (!((rows_w >> (row0 + j)) & 1u)) continue;
-                        const float v = e ? hi2(x[k]) : lo2(x[k]);
-                        uol[j * w] = (zero_in ? 0.f : tol[j * P]) + v;
-                        vmax = fmaxf(vmax, fabsf(v));
-                    }
-                }
-            }
+        float* up = u_out + ch * n + (size_t)(y0 + bt.r0) * w + x0 + bt.cl;
+        const ptrdiff_t us = bt.dr * (ptrdiff_t)w;
+        if constexpr (OV == 0) {
+            if (op.full)
+                block_write01<true>(x, tc, ts, zero_in, up, us, wx0 > 0.f, wx1 > 0.f, rows_w, vec,
+                                    vmax);
+            else
+                block_write01<false>(x, tc, ts, zero_in, up, us, wx0 > 0.f, wx1 > 0.f, rows_w, vec,
+                                     vmax);
         } else {
             // the weighted part of shared pixels is parked in the block's tile
             // for k_combine; the first contributor of a shared pixel (smallest
             // block index along each shared axis) also carries u_in, so the
             // combine pass only adds
-            const int first = shared_first(o), nsh = shared_per_seam(o);
-            const bool xfirst = !(kx > 0 && col >= first && col < first + nsh);
-            float* const mine = parked + ((size_t)blk * C + ch) * (B * B) + col;
+            const int first = shared_first(o), last = first + shared_per_seam(o);
+            const bool xf0 = !(kx > 0 && bt.cl >= first && bt.cl < last);
+            const bool xf1 = !(kx > 0 && bt.cl + 1 >= first && bt.cl + 1 < last);
+            float* const mine = parked + ((size_t)blk * C + ch) * (B * B) + bt.cl;
 #pragma unroll
-            for (int k = 0; k < NP; ++k) {
-#pragma unroll
-                for (int e = 0; e < 2; ++e) {
-                    const int ly = row0 + k + 8 * e;
-                    if (ly >= bh || !colok) continue;
-                    const float v = e ? hi2(x[k]) : lo2(x[k]);
-                    const float d = wx * s_wy[ly];
-                    const float uold = zero_in ? 0.f : tu[(ly + 1) * P + col + 1];
-                    if (d == 1.f) {
-                        uo[(size_t)(y0 + ly) * w + x0 + col] = uold + v;
-                    } else if (d > 0.f) {
-                        const bool yfirst = !(ky > 0 && ly >= first && ly < first + nsh);
-                        mine[ly * B] = (xfirst && yfirst) ? uold + d * v : d * v;
-                    }
-                    if (d > 0.f) vmax = fmaxf(vmax, fabsf(v));
+            for (int j = 0; j < 8; ++j) {
+                const int ly = bt.r0 + bt.dr * j;
+                const float wy = s_wy[ly];
+                const float d0 = wx0 * wy, d1 = wx1 * wy;
+                const float v0 = block_value(x, 0, j), v1 = block_value(x, 1, j);
+                const f2 u = zero_in ? 0ull : ld_pair<EV>(tc + j * ts);
+                const bool yf = !(ky > 0 && ly >= first && ly < last);
+                const float a = d0 == 1.f ? lo2(u) + v0 : (xf0 && yf) ? lo2(u) + d0 * v0 : d0 * v0;
+                const float b = d1 == 1.f ? hi2(u) + v1 : (xf1 && yf) ? hi2(u) + d1 * v1 : d1 * v1;
+                float* const dst = up + j * us;
+                float* const part = mine + ly * B;
+                float* const pa = d0 == 1.f ? dst : part;
+                if (d0 > 0.f && d1 > 0.f && (d0 == 1.f) == (d1 == 1.f) && (vec || d0 < 1.f)) {
+                    *reinterpret_cast<float2*>(pa) = make_float2(a, b);
+                } else {
+                    if (d0 > 0.f) pa[0] = a;
+                    if (d1 > 0.f) (d1 == 1.f ? dst : part)[1] = b;
                 }
+                if (d0 > 0.f) vmax = fmaxf(vmax, fabsf(v0));
+                if (d1 > 0.f) vmax = fmaxf(vmax, fabsf(v1));
             }
         }
         if (!more) break;
@@ -2477,22 +2718,20 @@ k_batch_grid(const BatchSeg* __restrict__ segs, int nseg, BatchState bs) {
 __global__ void __launch_bounds__(64, 8)
 k_batch_oras(const BatchSeg* __restrict__ segs, int nseg, int nunits, int o, float alpha,
              BatchState bs) {
-    constexpr int B = 32, NP = 8, TH = Smem2W::TH, P = Smem2W::PU, PB = Smem2W::PB;
+    constexpr int B = 32, TH = Smem2W::TH, P = Smem2W::PU, PB = Smem2W::PB;
     constexpr int TILE = Smem2W::USTRIDE;
     extern __shared__ float smem_raw[];
     float* const smem = reinterpret_cast<float*>(
         (reinterpret_cast<uintptr_t>(smem_raw) + 127) & ~static_cast<uintptr_t>(127));
     float* const s_u = smem;
-    float* const s_wy = smem + Smem2W::WY;
     float* const s_e = smem + Smem2W::EP;  // coarse patches of prolonging segments
     float* const s_b = smem + Smem2W::RHS_PRO;
-    __shared__ float s_red1[2], s_red2[2], s_seam[2][32];
+    __shared__ BlockShared sh;
     __shared__ __align__(8) unsigned long long s_bar[2];  // TMA tiles of buffer 0, 1
 
     const int t = threadIdx.x;
-    const int lane = t & 31, wi = t >> 5;
-    const int col = lane;
-    const int row0 = 16 * wi;
+    const BlockThread bt(t);
+    const int lane = bt.lane, wi = bt.wi;
     const int s = B - o;
     const float inv_o1 = o > 1 ? 1.f / (float)(o - 1) : 0.f;
     // whether a segment's tasks form their start by prolongation (uniform per task)
@@ -2555,7 +2794,7 @@ k_batch_oras(const BatchSeg* __restrict__ segs, int nseg, int nunits, int o, flo
             pend_tma |= 1u << bs_;
         } else if (!sg.zero_in) {
             const float* src = static_cast<const float*>(sg.in0) + tk.ch * n;
-            float* dst = s_u + bs_ * TILE;
+            float* dst = s_u + bs_ * TILE + 1;  // block column 0 at an 8-byte boundary
             const int gxa = px0 - 1 + lane, gxb = gxa + 32;
             const bool oka = gxa >= 0 && gxa < w;
             const bool okb = lane < TH - 32 && gxb < w;
@@ -2582,7 +2821,7 @@ k_batch_oras(const BatchSeg* __restrict__ segs, int nseg, int nunits, int o, flo
         }
         cp_async_commit();
         if (new_blk && lane < 16) {
-            const int gy = py0 + row0 + lane;
+            const int gy = py0 + 16 * wi + lane;
             if (gy < h) {
                 const uint32_t* row = sg.mbits + (size_t)gy * sg.wpr + (px0 >> 5);
                 nlo = __ldg(row);
@@ -2607,11 +2846,10 @@ k_batch_oras(const BatchSeg* __restrict__ segs, int nseg, int nunits, int o, flo
     prefetch(cur, 0, true);
     int buf = 0;
     int cur_seg = -1, cur_blk = -1;
-    f2 ndg[NP], keep[NP];
-    f2 ml2 = 0ull, mr2 = 0ull;
-    float wx = 0.f, dh = 0.f;
-    int x0 = 0, y0 = 0, bh = 0, kx = 0, ky = 0;
-    uint32_t rows_w = 0, mbk = 0;
+    BlockOp op;
+    float wx0 = 0.f, wx1 = 0.f;
+    int x0 = 0, y0 = 0;
+    uint32_t rows_w = 0;
     float vmax = 0.f, pmax = 0.f;
     unsigned* vmax_slot = nullptr;
     unsigned* pmax_slot = nullptr;
@@ -2661,162 +2899,55 @@ k_batch_oras(const BatchSeg* __restrict__ segs, int nseg, int nunits, int o, flo
         }
         if (cur.blk != cur_blk) {
             cur_blk = cur.blk;
-            kx = cur.blk % nbx;
-            ky = cur.blk / nbx;
+            const int kx = cur.blk % nbx, ky = cur.blk / nbx;
             x0 = kx * s;
             y0 = ky * s;
-            const int bw = min(B, w - x0);
-            bh = min(B, h - y0);
-            const uint32_t rowm = __funnelshift_r(mlo, mhi, x0 & 31);
-            uint32_t mb = 0;
-#pragma unroll
-            for (int rr = 0; rr < 16; ++rr) {
-                const uint32_t v = __shfl_sync(kFull, rowm, rr);
-                mb |= ((v >> col) & 1u) << rr;
-            }
-            const int gx = x0 + col;
-            const float hc = (col > 0 ? 1.f : (gx > 0 ? alpha : 0.f)) +
-                             (col + 1 < bw ? 1.f : (gx < w - 1 ? alpha : 0.f));
-            dh = (float)((gx > 0) + (gx < w - 1));
-            const float ml = col > 0 ? 1.f : 0.f, mr = col < B - 1 ? 1.f : 0.f;
-            ml2 = pk(ml, ml);
-            mr2 = pk(mr, mr);
-#pragma unroll
-            for (int k = 0; k < NP; ++k) {
-                float vc[2];
-#pragma unroll
-                for (int e = 0; e < 2; ++e) {
-                    const int ly = row0 + k + 8 * e, gy = y0 + ly;
-                    vc[e] = (ly > 0 ? 1.f : (gy > 0 ? alpha : 0.f)) +
-                            (ly + 1 < bh ? 1.f : (gy < h - 1 ? alpha : 0.f));
-                }
-                ndg[k] = pk(-(hc + vc[0]), -(hc + vc[1]));
-                keep[k] = pk(((mb >> k) & 1u) ? 0.f : 1.f, ((mb >> (k + 8)) & 1u) ? 0.f : 1.f);
-            }
-            mbk = mb;
-            wx = ramp_weight(col, kx, nbx, s, o, inv_o1);
-            const float wyl = ramp_weight(lane, ky, nby, s, o, inv_o1);
-            if (t < B) s_wy[t] = wyl;
-            rows_w = __ballot_sync(kFull, wyl > 0.f && lane < bh);
+            const int bh = min(B, h - y0);
+            block_operator(op, bt, __funnelshift_r(mlo, mhi, x0 & 31), x0, y0, min(B, w - x0), bh,
+                           w, h, alpha);
+            if (!op.full) clipped_diagonal(bt, y0, bh, h, alpha, sh.nv);
+            wx0 = x0 + bt.cl < w ? ramp_weight(bt.cl, kx, nbx, s, o, inv_o1) : 0.f;
+            wx1 = x0 + bt.cl + 1 < w ? ramp_weight(bt.cl + 1, kx, nbx, s, o, inv_o1) : 0.f;
+            rows_w = own_rows(bt, ky, nby, bh);
         }
         // TMA tiles start at the 4-aligned column below the halo column
-        const int du = sg.tma ? ((x0 - 1) & 3) : 0;
+        const int du = sg.tma ? ((x0 - 1) & 3) : 1;
         const int db = sg.tma ? (x0 & 3) : 0;
-        const float* tu = s_u + buf * TILE + du;
-        const float* tb = s_b + buf * Smem2W::BSTRIDE + db;
+        const float* tc = s_u + buf * TILE + du + (bt.r0 + 1) * P + bt.cl + 1;
+        const float* bc = s_b + buf * Smem2W::BSTRIDE + db + bt.r0 * PB + bt.cl;
+        const int ts = bt.dr * P, bs_b = bt.dr * PB;
         if (prolongs(sg)) {  // uniform per task
             const float* pe = s_e + buf * Smem2W::ESTRIDE;
             if (sg.pro_mode == 1)
-                prolong_into_tile<true>(s_u + buf * TILE + du, pe, row0, col, lane, wi, x0, y0,
-                                        mbk, hk, pmax);
+                prolong_into_tile<true>(s_u + buf * TILE + du, pe, bt, op, hk, pmax);
             else
-                prolong_into_tile<false>(s_u + buf * TILE + du, pe, row0, col, lane, wi, x0, y0,
-                                         mbk, hk, pmax);
+                prolong_into_tile<false>(s_u + buf * TILE + du, pe, bt, op, hk, pmax);
             __syncthreads();  // the residual reads the other threads' columns
         }
 
-        f2 x[NP], r[NP], p[NP], q[NP];
-        f2 acc0 = 0ull, acc1 = 0ull;
-#pragma unroll
-        for (int k = 0; k < NP; ++k) {
-            float rv[2];
-#pragma unroll
-            for (int e = 0; e < 2; ++e) {
-                const int ly = row0 + k + 8 * e, gy = y0 + ly;
-                float v = rhs_zero ? 0.f : tb[ly * PB + col];
-                if (!zero_in) {
-                    const float* c0 = tu + (ly + 1) * P + col + 1;
-                    const float dv = (float)((gy > 0) + (gy < h - 1));
-                    v = res_stencil<false>(v, dh + dv, c0[0], c0[-P], c0[P], c0[-1], c0[1]);
-                }
-                rv[e] = v;
-            }
-            r[k] = mul2(pk(rv[0], rv[1]), keep[k]);
-            p[k] = r[k];
-            x[k] = 0ull;
-            if (k & 1) acc1 = fma2(r[k], r[k], acc1);
-            else acc0 = fma2(r[k], r[k], acc0);
+        f2 x[8], r[8];
+        if (y0 > 0 && y0 + B < h) {
+            if (rhs_zero)
+                block_residual<false, true, true, true>(r, op, bt, tc, ts, bc, bs_b, zero_in, y0, h);
+            else
+                block_residual<false, false, true, true>(r, op, bt, tc, ts, bc, bs_b, zero_in, y0, h);
+        } else {
+            if (rhs_zero)
+                block_residual<false, true, false, true>(r, op, bt, tc, ts, bc, bs_b, zero_in, y0, h);
+            else
+                block_residual<false, false, false, true>(r, op, bt, tc, ts, bc, bs_b, zero_in, y0, h);
         }
-        acc0 = add2(acc0, acc1);
-        s_seam[wi][lane] = wi == 0 ? hi2(r[NP - 1]) : lo2(r[0]);
-        float part = warp_sum(lo2(acc0) + hi2(acc0));
-        if (lane == 0) s_red2[wi] = part;
-        __syncthreads();
-        float rr = s_red2[0] + s_red2[1];
-        float pb = s_seam[wi ^ 1][lane];
-        const float rtol2 = sg.rtol2;
-        const float rr_stop = rtol2 >= 0.f ? fmaxf(rtol2, 1e-14f) * rr
-                                           : fmaxf(1e-14f * rr, -rtol2);
-        const int iters = sg.iters;
-        for (int it = 0; it < iters; ++it) {
-            if (!(rr > rr_stop)) break;  // rr is identical in both warps
-            const f2 pu = wi == 0 ? pk(0.f, lo2(p[NP - 1])) : pk(pb, lo2(p[NP - 1]));
-            const f2 pd = wi == 0 ? pk(hi2(p[0]), pb) : pk(hi2(p[0]), 0.f);
-            acc0 = 0ull;
-            acc1 = 0ull;
-#pragma unroll
-            for (int k = 0; k < NP; ++k) {
-                const f2 left = __shfl_up_sync(kFull, p[k], 1);
-                const f2 right = __shfl_down_sync(kFull, p[k], 1);
-                const f2 up = k > 0 ? p[k - 1] : pu;
-                const f2 dn = k < NP - 1 ? p[k + 1] : pd;
-                f2 nbs = add2(up, dn);
-                nbs = fma2(ml2, left, nbs);
-                nbs = fma2(mr2, right, nbs);
-                const f2 qk = mul2(fma2(ndg[k], p[k], nbs), keep[k]);
-                q[k] = qk;
-                if (k & 1) acc1 = fma2(p[k], qk, acc1);
-                else acc0 = fma2(p[k], qk, acc0);
-            }
-            acc0 = add2(acc0, acc1);
-            part = warp_sum(lo2(acc0) + hi2(acc0));
-            if (lane == 0) s_red1[wi] = part;
-            __syncthreads();
-            const float pq = -(s_red1[0] + s_red1[1]);
-            if (!(pq > 0.f) || pq == INFINITY) break;
-            const float a = __fdividef(rr, pq);
-            const f2 a2 = pk(a, a);
-            acc0 = 0ull;
-            acc1 = 0ull;
-#pragma unroll
-            for (int k = 0; k < NP; ++k) {
-                x[k] = fma2(a2, p[k], x[k]);
-                r[k] = fma2(a2, q[k], r[k]);
-                if (k & 1) acc1 = fma2(r[k], r[k], acc1);
-                else acc0 = fma2(r[k], r[k], acc0);
-            }
-            acc0 = add2(acc0, acc1);
-            s_seam[wi][lane] = wi == 0 ? hi2(r[NP - 1]) : lo2(r[0]);
-            part = warp_sum(lo2(acc0) + hi2(acc0));
-            if (lane == 0) s_red2[wi] = part;
-            __syncthreads();
-            const float rrn = s_red2[0] + s_red2[1];
-            const float beta = __fdividef(rrn, rr);
-            rr = rrn;
-            const f2 b2 = pk(beta, beta);
-#pragma unroll
-            for (int k = 0; k < NP; ++k) p[k] = fma2(b2, p[k], r[k]);
-            pb = fmaf(beta, pb, s_seam[wi ^ 1][lane]);
-        }
+        block_cg(x, r, op, bt, sg.iters, sg.rtol2, sh);
 
-        // 0/1 weights: each pixel is written by the one block whose weight is
-        // 1 there, with u_in added
-        float* uo = static_cast<float*>(sg.out0) + cur.ch * n;
-        if (x0 + col < w && wx > 0.f) {
-            float* uol = uo + (size_t)(y0 + row0) * w + x0 + col;
-            const float* tol = tu + (row0 + 1) * P + col + 1;
-#pragma unroll
-            for (int e = 0; e < 2; ++e) {
-#pragma unroll
-                for (int k = 0; k < NP; ++k) {
-                    const int j = k + 8 * e;
-                    if (!((rows_w >> (row0 + j)) & 1u)) continue;
-                    const float v = e ? hi2(x[k]) : lo2(x[k]);
-                    uol[(size_t)j * w] = (zero_in ? 0.f : tol[j * P]) + v;
-                    vmax = fmaxf(vmax, fabsf(v));
-                }
-            }
-        }
+        float* uo = static_cast<float*>(sg.out0);
+        const bool vec = (w & 1) == 0 && (reinterpret_cast<uintptr_t>(uo) & 7) == 0;
+        float* up = uo + cur.ch * n + (size_t)(y0 + bt.r0) * w + x0 + bt.cl;
+        const ptrdiff_t us = bt.dr * (ptrdiff_t)w;
+        if (op.full)
+            block_write01<true>(x, tc, ts, zero_in, up, us, wx0 > 0.f, wx1 > 0.f, rows_w, vec, vmax);
+        else
+            block_write01<false>(x, tc, ts, zero_in, up, us, wx0 > 0.f, wx1 > 0.f, rows_w, vec,
+                                 vmax);
         if (!more) break;
         g = g2;
         cur = nxt;
@@ -3060,7 +3191,7 @@ cudaError_t launch_oras_2w(const float* u_in, int zero_in, const float* rhs, int
     int nsm = 0, oc = 0;
     size_t smem = 0;
     const void* kern = nullptr;
-    decltype(&k_oras_2w<false, 0, false>) fn = nullptr;  // the FP32 kernel
+    decltype(&k_oras_2w<false, 0, 0>) fn = nullptr;  // the FP32 kernel
     CUtensorMap tm_u, tm_b, tm_e;
     std::memset(&tm_u, 0, sizeof tm_u);
     std::memset(&tm_b, 0, sizeof tm_b);
@@ -3073,11 +3204,14 @@ cudaError_t launch_oras_2w(const float* u_in, int zero_in, const float* rhs, int
         use_tma_e = use_tma && pm != 0 &&
                     make_map(&tm_e, pro_e, wH, hH, C, Smem2W::EPW, Smem2W::EH);
         smem = Smem2W::bytes(!rhs_zero, pm != 0);
-#define DI_ORAS_SEL(SH)                                                                \
-    (pm == 1   ? (f64 ? k_oras_2w<true, 1, SH> : k_oras_2w<false, 1, SH>)               \
-     : pm == 2 ? (f64 ? k_oras_2w<true, 2, SH> : k_oras_2w<false, 2, SH>)               \
-               : (f64 ? k_oras_2w<true, 0, SH> : k_oras_2w<false, 0, SH>))
-        fn = shared_per_seam(o) > 0 ? DI_ORAS_SEL(true) : DI_ORAS_SEL(false);
+#define DI_ORAS_SEL(OV)                                                               \
+    (pm == 1   ? (f64 ? k_oras_2w<true, 1, OV> : k_oras_2w<false, 1, OV>)              \
+     : pm == 2 ? (f64 ? k_oras_2w<true, 2, OV> : k_oras_2w<false, 2, OV>)              \
+               : (f64 ? k_oras_2w<true, 0, OV> : k_oras_2w<false, 0, OV>))
+        fn = o == 2          ? DI_ORAS_SEL(0)
+             : (o & 1) == 0  ? DI_ORAS_SEL(1)
+             : f64           ? k_oras_2w<true, 0, 2>  // no fused prolongation (prolong_fusable)
+                             : k_oras_2w<false, 0, 2>;
 #undef DI_ORAS_SEL
         kern = (const void*)fn;
         oc = cached_occupancy(kern, 64, smem, Smem2W::bytes(true, pm != 0), &nsm);

@@ -269,6 +269,25 @@ def test_transfers_vector_and_scalar_paths_agree(di, h, w):
     assert np.array_equal(pa, pb)
 
 
+@pytest.mark.parametrize("h", [5, 31, 32, 33, 61, 62, 63, 77])
+@pytest.mark.parametrize("w,o", [(96, 2), (95, 2), (64, 1), (70, 5), (62, 16), (33, 4)])
+def test_oras_block_edges(di, h, w, o):
+    # blocks clipped at every remainder of the block height, odd strides (tile
+    # columns off 8-byte boundaries) and outputs off 8-byte boundaries: against
+    # the oracle's K-step CG (the bound of test_oras_iteration_matches_oracle_cg)
+    # and the same bits wherever u_out lies
+    f, fn, c = _case(h, w, 2, 0.07, 7 * h + w + o)
+    g = np.random.default_rng(h + w)
+    u = np.where(c.astype(bool), f, g.uniform(0, 255, f.shape)).astype(np.float32)
+    with di.Context(block=32, overlap=o, alpha=0.4) as ctx:
+        out = N(ctx.oras_iteration(T(u), T(fn), T(c), 6, rhs_zero=True))
+        ref = M.oras_iteration(u, M.rhs(f, c), c, 32, o, 0.4, ("cg", 6))
+        assert np.abs(out - ref).max() < 1e-3 * np.abs(ref - u).max() + 2e-4
+        off = _unaligned(np.zeros_like(u))
+        assert np.array_equal(N(ctx.oras_iteration(T(u), T(fn), T(c), 6, rhs_zero=True, out=off)),
+                              out)
+
+
 PRO_CASES = [  # (h, w, overlap, rhs_zero, aligned)
     (70, 96, 2, True, True), (70, 96, 2, False, False), (70, 96, 6, False, True),
     (33, 35, 2, False, True), (130, 100, 2, True, False), (61, 250, 6, True, True),
