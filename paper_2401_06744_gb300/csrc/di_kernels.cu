@@ -945,6 +945,53 @@ k_pack_mask(const uint8_t* __restrict__ c, int w, int h, uint32_t* __restrict__ 
     pack_mask_body(c, w, h, bits, wpr, unknown, blockIdx.x, gridDim.x);
 }
 
+// The same for rows of whole 16-byte groups (w a multiple of 16, aligned
+// base): a thread turns 16 mask bytes into half a word, and two threads make
+// one.  3840x2160 (8.3 MB, 1.2 us at the copy rate): a byte per lane and a
+// ballot per word, with a division per word, took 21.7 us; an iteration with
+// its packing at that size went from 213 to 195 us.
+__global__ void __launch_bounds__(256)
+k_pack_mask16(const uint8_t* __restrict__ c, int w, int h, uint32_t* __restrict__ bits, int wpr,
+              unsigned long long* __restrict__ unknown) {
+    const int halves = 2 * wpr, groups = w >> 4;  // half words per row, those inside the image
+    const int x = blockIdx.x * 32 + threadIdx.x;  // half word of the row
+    unsigned unk = 0;
+    const int y0 = ((int)blockIdx.y * 8 + (int)threadIdx.y) * 4;
+    uint4 v[4];
+#pragma unroll
+    for (int r = 0; r < 4; ++r)
+        if (x < groups && y0 + r < h)
+            v[r] = __ldg(reinterpret_cast<const uint4*>(c + (size_t)(y0 + r) * w) + x);
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+        unsigned half = 0xffffu;
+        if (x < groups && y0 + r < h) {
+            // per byte 0 or 1, then the four flags of a word gathered at bit 24
+            const unsigned f0 = __vminu4(v[r].x, 0x01010101u) * 0x01020408u;
+            const unsigned f1 = __vminu4(v[r].y, 0x01010101u) * 0x01020408u;
+            const unsigned f2_ = __vminu4(v[r].z, 0x01010101u) * 0x01020408u;
+            const unsigned f3 = __vminu4(v[r].w, 0x01010101u) * 0x01020408u;
+            half = ((f0 >> 24) & 15u) | ((f1 >> 20) & 0xf0u) | ((f2_ >> 16) & 0xf00u) |
+                   ((f3 >> 12) & 0xf000u);
+            unk += 16u - (unsigned)__popc(half);
+        }
+        const unsigned other = __shfl_xor_sync(kFull, half, 1);
+        if (!(x & 1) && x < halves && y0 + r < h)
+            bits[(size_t)(y0 + r) * wpr + (x >> 1)] = half | (other << 16);
+    }
+    if (unknown) {
+        __shared__ unsigned s_u[8];
+        const unsigned t = __reduce_add_sync(kFull, unk);
+        if (threadIdx.x == 0) s_u[threadIdx.y] = t;
+        __syncthreads();
+        if (threadIdx.x == 0 && threadIdx.y == 0) {
+            unsigned long long a = 0;
+            for (int i = 0; i < 8; ++i) a += s_u[i];
+            if (a) atomicAdd(unknown, a);
+        }
+    }
+}
+
 // One ORAS iteration, one warp per (block, channel) task.
 //
 // Lane layout: lane = (g, col), col = lane % B the block column and g the row
@@ -3634,6 +3681,13 @@ cudaError_t launch_pack_mask(const uint8_t* c, int w, int h, uint32_t* bits,
     const int wpr = mask_words_per_row(w);
     const long long words = (long long)h * wpr;
     if (words > 0x7fffffffLL) return cudaErrorInvalidValue;
+    const unsigned rows32 = (unsigned)((h + 31) / 32);
+    if (w % 16 == 0 && (reinterpret_cast<uintptr_t>(c) & 15) == 0 && rows32 <= 65535u) {
+        k_pack_mask16<<<dim3((unsigned)((2 * wpr + 31) / 32), rows32), dim3(32, 8), 0, s>>>(
+            c, w, h, bits, wpr, unknown);
+        count();
+        return cudaGetLastError();
+    }
     long long blocks = (words + 31) / 32;  // 8 warps x 4 words per CTA pass
     if (blocks > 152 * 8) blocks = 152 * 8;
     if (blocks < 1) blocks = 1;
