@@ -608,13 +608,16 @@ __device__ __forceinline__ void restrict_body(const TU* __restrict__ u, const TB
     const int ch = bz;
     if (X >= wH || Y >= hH) return;
     const size_t n = (size_t)w * h, nH = (size_t)wH * hH, P = (size_t)Y * wH + X;
-    if (cH[P]) { stf(rH + ch * nH + P, 0.f); return; }
+    const uint8_t known = cH[P];
     const TU* uc = u + ch * n;
     const int x0 = 2 * X - 1, y0 = 2 * Y - 1;
     if (VEC && X >= 1 && Y >= 1 && 2 * X + 2 < w && 2 * Y + 2 < h) {
         // a cell whose 4x4 patch lies inside the image (all but the border
         // cells): every child has four neighbours and the count is 4, so the
-        // same sums as below without a bounds test (the same bits)
+        // same sums as below without a bounds test (the same bits).  The
+        // patch is loaded beside the cell's mask byte, not after it: the
+        // kernel waits for memory, and known cells, whose sum is dropped, are
+        // few and their rows are the neighbours' rows too
         const TU* r0 = uc + (size_t)y0 * w + x0;
         float t[4][4];
 #pragma unroll
@@ -639,9 +642,10 @@ __device__ __forceinline__ void restrict_body(const TU* __restrict__ u, const TB
                 sum += rhs - lu;
             }
         }
-        stf(rH + ch * nH + P, (float)sum);
+        stf(rH + ch * nH + P, known ? 0.f : (float)sum);
         return;
     }
+    if (known) { stf(rH + ch * nH + P, 0.f); return; }
     float t[4][4];
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
@@ -690,6 +694,63 @@ __device__ __forceinline__ void restrict_body(const TU* __restrict__ u, const TB
     // 4 sum / cnt with cnt in {1, 2, 4} (children inside the image): an exact
     // power-of-two scaling, so a multiplication gives the quotient bit for bit
     stf(rH + ch * nH + P, (float)(sum * (R)(4 >> (cnt >> 1))));
+}
+
+// The large levels of FP32 images of several channels: one thread per coarse
+// cell and all its channels, every channel's patch in flight together.  The
+// kernel waits for memory, so what counts is loads in flight: CTAs of 128
+// threads, eight per SM at 64 registers (a few spilled: still better than three
+// CTAs of 256 at 77 registers, 34.5 us).  3840x2160 RGB (127 MB, 19 us at the
+// copy rate): 41.1 us with a thread per cell and channel and the patch loaded
+// after the mask byte, 36.8 loaded beside it, 28.9 here; with a right-hand side
+// 49 and 39.7.  VEC: children pairs as 8-byte words.  Border cells as above.
+template <int C, bool VEC>
+__global__ void __launch_bounds__(128, 8)
+k_restrict_c(const float* __restrict__ u, const float* __restrict__ b, int rhs_zero, int w, int h,
+             const uint8_t* __restrict__ cH, float* __restrict__ rH, int wH, int hH) {
+    const int X = blockIdx.x * 32 + threadIdx.x, Y = blockIdx.y * 4 + threadIdx.y;
+    if (X >= wH || Y >= hH) return;
+    const size_t n = (size_t)w * h, nH = (size_t)wH * hH, P = (size_t)Y * wH + X;
+    if (X < 1 || Y < 1 || 2 * X + 2 >= w || 2 * Y + 2 >= h) {
+        for (int ch = 0; ch < C; ++ch)
+            restrict_body<VEC, float, float, float, false>(u, b, rhs_zero, w, h, cH, rH, wH, hH,
+                                                           blockIdx.x, blockIdx.y, ch);
+        return;
+    }
+    const uint8_t known = cH[P];
+    auto pair = [](const float* p) {
+        return VEC ? *reinterpret_cast<const float2*>(p) : make_float2(p[0], p[1]);
+    };
+    float2 mid[C][4], rb[C][2];
+    float l[C][2], r[C][2];
+    const size_t at = (size_t)(2 * Y - 1) * w + 2 * X;  // row above the children, left child
+#pragma unroll
+    for (int ch = 0; ch < C; ++ch) {
+        const float* p = u + ch * n + at;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) mid[ch][j] = pair(p + (size_t)j * w);
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+            l[ch][j] = p[(size_t)(j + 1) * w - 1];
+            r[ch][j] = p[(size_t)(j + 1) * w + 2];
+            rb[ch][j] = make_float2(0.f, 0.f);
+            if (!rhs_zero) rb[ch][j] = pair(b + ch * n + at + (size_t)(j + 1) * w);
+        }
+    }
+#pragma unroll
+    for (int ch = 0; ch < C; ++ch) {
+        // the sums of restrict_body's interior path, in its order
+        float sum = 0.f;
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+            const float2 up = mid[ch][j], ce = mid[ch][j + 1], dn = mid[ch][j + 2];
+            const float l0 = 4.f * ce.x - (l[ch][j] + ce.y + up.x + dn.x);
+            const float l1 = 4.f * ce.y - (ce.x + r[ch][j] + up.y + dn.y);
+            sum += (rhs_zero ? 0.f : rb[ch][j].x) - l0;
+            sum += (rhs_zero ? 0.f : rb[ch][j].y) - l1;
+        }
+        rH[ch * nH + P] = known ? 0.f : sum;
+    }
 }
 
 template <bool VEC, class TU, class TB, class TO, bool F64>
@@ -2755,11 +2816,19 @@ k_batch_grid(const BatchSeg* __restrict__ segs, int nseg, BatchState bs) {
         values_down_body(static_cast<const uint8_t*>(sg.in0), static_cast<const float*>(sg.in1),
                          w, h, sg.C, static_cast<const uint8_t*>(sg.in2),
                          static_cast<float*>(sg.out0), wH, hH, sg.mode, bx, by);
-    else if (KIND == kBRestrict)
-        restrict_body<false, float, float, float, false>(
-            static_cast<const float*>(sg.in0), static_cast<const float*>(sg.in1), sg.rhs_zero, w,
-            h, static_cast<const uint8_t*>(sg.in2), static_cast<float*>(sg.out0), wH, hH, bx, by,
-            bz);
+    else if (KIND == kBRestrict) {
+        const float* u = static_cast<const float*>(sg.in0);
+        const float* b = static_cast<const float*>(sg.in1);
+        const uint8_t* cH = static_cast<const uint8_t*>(sg.in2);
+        float* rH = static_cast<float*>(sg.out0);
+        if ((w & 1) == 0 && ((reinterpret_cast<uintptr_t>(u) |
+                              (sg.rhs_zero ? 0 : reinterpret_cast<uintptr_t>(b))) & 7) == 0)
+            restrict_body<true, float, float, float, false>(u, b, sg.rhs_zero, w, h, cH, rH, wH,
+                                                            hH, bx, by, bz);
+        else
+            restrict_body<false, float, float, float, false>(u, b, sg.rhs_zero, w, h, cH, rH, wH,
+                                                             hH, bx, by, bz);
+    }
     else if (KIND == kBProlong)
         prolong_body<false, float, float>(static_cast<const float*>(sg.in0), wH, hH,
                                           static_cast<const float*>(sg.in1),
@@ -3521,7 +3590,17 @@ cudaError_t launch_restrict(const float* u, const float* b, int rhs_zero, const 
     const bool vec = su == kF32 && sb == kF32 && (w % 2 == 0) &&
                      ((reinterpret_cast<uintptr_t>(u) |
                        reinterpret_cast<uintptr_t>(rhs_zero ? nullptr : b)) % 8 == 0);
-    if (su == kF32 && sb == kF32 && sr == kF32) {
+    // one thread for all channels of a cell where the level's cells still fill the
+    // GPU's threads (at 960x540 cells both forms take 10.3 us, at 1920x1080 28.9
+    // against 36.8)
+    if (su == kF32 && sb == kF32 && sr == kF32 && !f64 && C > 1 &&
+        (long long)wH * hH >= 152LL * 2048) {
+        const dim3 b1(32, 4), g1 = grid2(wH, hH, b1);
+        auto* const kern = C == 2   ? (vec ? k_restrict_c<2, true> : k_restrict_c<2, false>)
+                           : C == 3 ? (vec ? k_restrict_c<3, true> : k_restrict_c<3, false>)
+                                    : (vec ? k_restrict_c<4, true> : k_restrict_c<4, false>);
+        kern<<<g1, b1, 0, s>>>(u, b, rhs_zero, w, h, cH, rH, wH, hH);
+    } else if (su == kF32 && sb == kF32 && sr == kF32) {
         if (vec && f64)
             k_restrict<true, float, float, float, true><<<grid, blk, 0, s>>>(
                 u, b, rhs_zero, w, h, cH, rH, wH, hH);
