@@ -19,7 +19,9 @@
 //   k_oras_2w        Algorithm 2 steps 1-3 for 32x32 blocks: two warps per (block,
 //                    channel), plain CG in registers as packed FP32 pairs, tiles by
 //                    TMA; optionally the start formed by prolongation inside it
-//   k_oras_2w_h      the same with FP16 / BF16 local iterates
+//   k_oras_4w        the same with four warps per (block, channel), for launches of
+//                    few local problems (the same bits)
+//   k_oras_2w_h      k_oras_2w with FP16 / BF16 local iterates
 //   k_oras_warp      8x8 and 16x16 blocks: one warp per (block, channel)
 //   k_combine        Algorithm 2 step 3 for pixels shared by several blocks: the
 //                    sums of their weighted contributions in a fixed order
@@ -1594,6 +1596,14 @@ __device__ __forceinline__ float quotient(float a, float b) {
     return a * r;
 }
 
+// Sum over a warp of the two-warp form, the row groups last, so that the
+// four-warp form (a warp per row group) adds in the same order.
+__device__ __forceinline__ float warp_sum_block(float v) {
+#pragma unroll
+    for (int d = 8; d > 0; d >>= 1) v += __shfl_xor_sync(kFull, v, d);
+    return v + __shfl_xor_sync(kFull, v, 16);
+}
+
 // Up to `iters` CG steps on A_i x = r from x = 0 (r is overwritten); both
 // warps of the block.  rtol2 >= 0: relative stop (r.r <= max(rtol2, 1e-14)
 // (r.r)_0); rtol2 < 0: also stop once r.r <= -rtol2 (an absolute level, or the
@@ -1619,7 +1629,7 @@ __device__ __forceinline__ unsigned block_cg_t(f2 (&x)[8], f2 (&r)[8], const Blo
     }
     acc0 = add2(acc0, acc1);
     if (bt.g) sh.seam[bt.wi][bt.l] = make_float2(lo2(r[0]), lo2(r[4]));
-    float part = warp_sum(lo2(acc0) + hi2(acc0));
+    float part = warp_sum_block(lo2(acc0) + hi2(acc0));
     if (bt.lane == 0) sh.red2[bt.wi] = part;
     __syncthreads();
     float rr = sh.red2[0] + sh.red2[1];
@@ -1671,7 +1681,7 @@ __device__ __forceinline__ unsigned block_cg_t(f2 (&x)[8], f2 (&r)[8], const Blo
             acc1 = k ? fma2(p[4 + k], q[4 + k], acc1) : mul2(p[4 + k], q[4 + k]);
         }
         acc0 = add2(acc0, acc1);
-        part = warp_sum(lo2(acc0) + hi2(acc0));
+        part = warp_sum_block(lo2(acc0) + hi2(acc0));
         if (bt.lane == 0) sh.red1[bt.wi] = part;
         __syncthreads();
         const float pq = -(sh.red1[0] + sh.red1[1]);
@@ -1694,7 +1704,7 @@ __device__ __forceinline__ unsigned block_cg_t(f2 (&x)[8], f2 (&r)[8], const Blo
         }
         acc0 = add2(acc0, acc1);
         if (bt.g) sh.seam[bt.wi][bt.l] = make_float2(lo2(r[0]), lo2(r[4]));
-        part = warp_sum(lo2(acc0) + hi2(acc0));
+        part = warp_sum_block(lo2(acc0) + hi2(acc0));
         if (bt.lane == 0) sh.red2[bt.wi] = part;
         __syncthreads();
         const float rrn = sh.red2[0] + sh.red2[1];
@@ -1731,6 +1741,13 @@ __device__ __forceinline__ uint32_t own_rows(const BlockThread& bt, int ky, int 
 // Local row j of column c of a solution.
 __device__ __forceinline__ float block_value(const f2 (&x)[8], int c, int j) {
     return j < 4 ? lo2(x[4 * c + j]) : hi2(x[4 * c + j - 4]);
+}
+
+// What a block of weight d stores of a pixel: u_in + v where the pixel is its
+// own (d = 1), its weighted part elsewhere, the first contributor's with u_in.
+// Every rounding explicit, so that each block kernel gets the same bits.
+__device__ __forceinline__ float shared_part(float d, float v, float u, bool first) {
+    return d == 1.f || first ? __fmaf_rn(d, v, u) : __fmul_rn(d, v);
 }
 
 // The write of 0/1 weights (overlap 2): each pixel is written by the one block
@@ -1844,14 +1861,14 @@ __device__ __forceinline__ void prolong_into_tile(float* tw, const float* pe,
     }
 }
 
-// The coarse cells a task's prolongation reads, by 4-byte cp.async (all 64
+// The coarse cells a task's prolongation reads, by 4-byte cp.async (all nt
 // threads): rows (py0 >> 1) - 1 + r and columns (px0 >> 1) - 1 + q, r, q <
 // 18, each clamped to the level as the prolongation clamps its indices,
 // into dst with pitch Smem2W::EPW.  The caller commits the group.
 __device__ __forceinline__ void copy_patch_clamped(float* dst, const float* e, int px0, int py0,
-                                                   int wH, int hH, int t) {
+                                                   int wH, int hH, int t, int nt = 64) {
     const int Ys = (py0 >> 1) - 1, Xs = (px0 >> 1) - 1;
-    for (int i = t; i < Smem2W::ES; i += 64) {
+    for (int i = t; i < Smem2W::ES; i += nt) {
         const int r = i / Smem2W::EW, q = i - r * Smem2W::EW;
         const int Y = min(max(Ys + r, 0), hH - 1), X = min(max(Xs + q, 0), wH - 1);
         cp_async4(dst + r * Smem2W::EPW + q, e + (size_t)Y * wH + X, true);
@@ -2214,8 +2231,8 @@ k_oras_2w(const float* __restrict__ u_in, int zero_in, const float* __restrict__
                 const float v0 = block_value(x, 0, j), v1 = block_value(x, 1, j);
                 const f2 u = zero_in ? 0ull : ld_pair<EV>(tc + j * ts);
                 const bool yf = !(ky > 0 && ly >= first && ly < last);
-                const float a = d0 == 1.f ? lo2(u) + v0 : (xf0 && yf) ? lo2(u) + d0 * v0 : d0 * v0;
-                const float b = d1 == 1.f ? hi2(u) + v1 : (xf1 && yf) ? hi2(u) + d1 * v1 : d1 * v1;
+                const float a = shared_part(d0, v0, lo2(u), xf0 && yf);
+                const float b = shared_part(d1, v1, hi2(u), xf1 && yf);
                 float* const dst = up + j * us;
                 float* const part = mine + ly * B;
                 float* const pa = d0 == 1.f ? dst : part;
@@ -2245,6 +2262,352 @@ k_oras_2w(const float* __restrict__ u_in, int zero_in, const float* __restrict__
     }
 }
 
+
+// ---- four warps per block: the same iteration where few blocks are to be solved
+//
+// On the small levels of a decode a launch has fewer local problems than the
+// GPU has SMs and lasts as long as one of them: about 6 us at ten steps, a warp
+// issuing an instruction every 4 cycles in the CG steps and every 6 to 9 in the
+// code around them, which runs once and cold.  So this form gives each problem
+// twice the threads and every thread half the work: warp 2 wi + g takes row
+// group g of warp wi of the two-warp form (BlockThread), lane = column, one
+// column of eight rows (four packed pairs) per thread.  One CTA per problem, no
+// prefetch.  Every sum is formed in the order of the two-warp form, so the bits
+// are the same and the launcher may choose by the number of problems alone.
+// With every SM busy it is the slower one (a barrier and a sum more per pixel).
+// 256x256 decode 249 -> 211 us, 481x321 RGB (overlap 6) 432 -> 394, 1920x1080 RGB
+// 1115 -> 1090, 3840x2160 RGB 1606 -> 1589.
+template <int PRO, int OV>
+__global__ void __launch_bounds__(128)
+k_oras_4w(const float* __restrict__ u_in, int zero_in, const float* __restrict__ rhs, int rhs_zero,
+          const uint32_t* __restrict__ mbits, int wpr, int w, int h, int C, int o, int nbx, int nby,
+          float alpha, int iters, float rtol2, float* __restrict__ u_out,
+          float* __restrict__ parked, unsigned* __restrict__ maxupd,
+          const __grid_constant__ CUtensorMap tm_u, const __grid_constant__ CUtensorMap tm_b,
+          int use_tma, unsigned* __restrict__ errflag,
+          unsigned long long* __restrict__ step_count, const float* __restrict__ eH, int wH,
+          int hH, unsigned* __restrict__ maxpro, const __grid_constant__ CUtensorMap tm_e,
+          int use_tma_e) {
+    constexpr int B = 32, TH = Smem2W::TH, P = Smem2W::PU, PB = Smem2W::PB;
+    constexpr int EW = Smem2W::EPW;
+    __shared__ __align__(128) float s_u[Smem2W::USTRIDE];
+    __shared__ __align__(128) float s_b[Smem2W::BSTRIDE];
+    __shared__ __align__(128) float s_e[PRO ? Smem2W::ESTRIDE : 32];
+    __shared__ float s_wy[B], s_row0[2][32], s_row7[4][32];
+    __shared__ float4 s_red1, s_red2;
+    __shared__ __align__(8) unsigned long long s_bar;
+
+    const int t = threadIdx.x, lane = t & 31, wrp = t >> 5;
+    const int wi = wrp >> 1, g = wrp & 1;
+    const int r0 = wi ? (g ? 16 : 31) : (g ? 15 : 0), dr = wi == g ? 1 : -1;
+    const int s = B - o;
+    const int blk = (int)blockIdx.x / C, ch = (int)blockIdx.x - blk * C;
+    const int ky = blk / nbx, kx = blk - ky * nbx, x0 = kx * s, y0 = ky * s;
+    const size_t n = (size_t)w * h;
+    const unsigned bar = (unsigned)__cvta_generic_to_shared(&s_bar);
+
+    // the tiles: one TMA box each, or 4-byte cp.async, as in k_oras_2w
+    if (use_tma) {
+        if (t == 0) {
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar) : "memory");
+            asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+            const unsigned bytes = (zero_in ? 0u : (unsigned)Smem2W::TMA_U_BYTES) +
+                                   (rhs_zero ? 0u : (unsigned)Smem2W::TMA_B_BYTES) +
+                                   (PRO != 0 && use_tma_e ? (unsigned)Smem2W::TMA_E_BYTES : 0u);
+            asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;"
+                         :: "r"(bar), "r"(bytes) : "memory");
+            if (!zero_in)
+                tma_load_3d((unsigned)__cvta_generic_to_shared(s_u), &tm_u, (x0 - 1) & ~3, y0 - 1,
+                            ch, bar);
+            if (!rhs_zero)
+                tma_load_3d((unsigned)__cvta_generic_to_shared(s_b), &tm_b, x0 & ~3, y0, ch, bar);
+            if (PRO != 0 && use_tma_e)
+                tma_load_3d((unsigned)__cvta_generic_to_shared(s_e), &tm_e,
+                            ((x0 >> 1) - 1) & ~3, (y0 >> 1) - 1, ch, bar);
+        }
+    } else {
+        if (!zero_in) {
+            const float* src = u_in + ch * n;
+            const int gxa = x0 - 1 + lane, gxb = gxa + 32;
+            const bool oka = gxa >= 0 && gxa < w, okb = lane < TH - 32 && gxb < w;
+            for (int ty = wrp; ty < TH; ty += 4) {
+                const int gy = y0 - 1 + ty;
+                const bool rok = gy >= 0 && gy < h;
+                const float* row = src + (ptrdiff_t)gy * w;
+                float* dst = s_u + ty * P + 1;
+                cp_async4(dst + lane, (rok && oka) ? row + gxa : src, rok && oka);
+                if (lane < TH - 32)
+                    cp_async4(dst + lane + 32, (rok && okb) ? row + gxb : src, rok && okb);
+            }
+        }
+        if (!rhs_zero) {
+            const float* src = rhs + ch * n;
+            const int gx = x0 + lane;
+            for (int ly = wrp; ly < B; ly += 4) {
+                const int gy = y0 + ly;
+                const bool ok = gx < w && gy < h;
+                cp_async4(s_b + ly * PB + lane, ok ? src + (size_t)gy * w + gx : src, ok);
+            }
+        }
+    }
+    if (PRO != 0 && !use_tma_e)
+        copy_patch_clamped(s_e, eH + (size_t)ch * wH * hH, x0, y0, wH, hH, t, 128);
+    cp_async_commit();
+
+    // mask bits: lane j < 8 the row of local row j; with a prolongation, the
+    // thread's pixel of the halo (warp: above, below, left, right)
+    uint32_t rowm = 0xffffffffu;
+    {
+        const int gy = y0 + r0 + dr * lane;
+        if (lane < 8 && gy < h) {
+            const uint32_t* row = mbits + (size_t)gy * wpr + (x0 >> 5);
+            rowm = __funnelshift_r(__ldg(row), __ldg(row + 1), x0 & 31);
+        }
+    }
+    bool hkn = true;  // known or off the image
+    if (PRO != 0) {
+        const int hy = wrp == 0 ? y0 - 1 : wrp == 1 ? y0 + B : y0 + lane;
+        const int hx = wrp < 2 ? x0 + lane : wrp == 2 ? x0 - 1 : x0 + B;
+        if (hx >= 0 && hx < w && hy >= 0 && hy < h)
+            hkn = (__ldg(mbits + (size_t)hy * wpr + (hx >> 5)) >> (hx & 31)) & 1u;
+    }
+
+    // the local operator of the thread's column (block_operator's values)
+    const int bw = min(B, w - x0), bh = min(B, h - y0);
+    const int gx = x0 + lane;
+    const float hc = (lane > 0 ? 1.f : (gx > 0 ? alpha : 0.f)) +
+                     (lane + 1 < bw ? 1.f : (gx < w - 1 ? alpha : 0.f));
+    f2 nd[4], keep[4];
+    uint32_t own = 0;  // bit j: local row j in the image
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        float d[2], kp[2];
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+            const int j = k + 4 * e, ly = r0 + dr * j, gy = y0 + ly;
+            const float vc = (ly > 0 ? 1.f : (gy > 0 ? alpha : 0.f)) +
+                             (ly + 1 < bh ? 1.f : (gy < h - 1 ? alpha : 0.f));
+            d[e] = -(hc + vc);
+            kp[e] = ((__shfl_sync(kFull, rowm, j) >> lane) & 1u) ? 0.f : 1.f;
+            if (ly < bh) own |= 1u << j;
+        }
+        nd[k] = pk(d[0], d[1]);
+        keep[k] = pk(kp[0], kp[1]);
+    }
+    const int odd = lane & 1, outer = odd ? lane + 1 : lane - 1;
+    const float mo = (lane == 0 || lane == 31) ? 0.f : 1.f;  // the outer column is in the block
+    const f2 mo2 = pk(mo, mo);
+    const float inv_o1 = o > 1 ? 1.f / (float)(o - 1) : 0.f;
+    const float wx = gx < w ? ramp_weight(lane, kx, nbx, s, o, inv_o1) : 0.f;
+    if (OV != 0 && t < B) s_wy[t] = lane < bh ? ramp_weight(lane, ky, nby, s, o, inv_o1) : 0.f;
+
+    cp_async_wait_all();
+    __syncthreads();  // the mbarrier is initialised, the cp.async tiles are there
+    if (use_tma) {
+        const bool ok = mbar_wait(bar, 0u);
+        if (__syncthreads_or(!ok)) {
+            if (!ok) mbar_wait(bar, 0u);  // one more bounded wait before the CTA leaves
+            if (t == 0 && errflag) atomicExch(errflag, 1u);
+            return;
+        }
+    }
+    const int du = use_tma ? ((x0 - 1) & 3) : 1, db = use_tma ? (x0 & 3) : 0;
+    float* const tc = s_u + du + (r0 + 1) * P + lane + 1;  // local row 0
+    const int ts = dr * P;
+    float pmax = 0.f;
+    if constexpr (PRO != 0) {
+        const int Ys = (y0 >> 1) - 1, Xs = (x0 >> 1) - 1;
+        float* const pw = s_e + (use_tma_e ? Xs - (Xs & ~3) : 0);
+        if (use_tma_e && (Ys < 0 || Xs < 0 || Ys + Smem2W::EW > hH || Xs + Smem2W::EW > wH)) {
+            // cells off the level take the value of their clamped cell
+            for (int i = t; i < Smem2W::ES; i += 128) {
+                const int r = i / Smem2W::EW, q = i - r * Smem2W::EW;
+                const int Yc = min(max(Ys + r, 0), hH - 1), Xc = min(max(Xs + q, 0), wH - 1);
+                if (Yc != Ys + r || Xc != Xs + q) pw[r * EW + q] = pw[(Yc - Ys) * EW + (Xc - Xs)];
+            }
+            __syncthreads();  // block-uniform branch
+        }
+        // the start of the iteration in the tile, as in prolong_into_tile
+        const int es = dr * EW;
+        const float* pr = pw + (1 + (r0 >> 1)) * EW + 1 + (lane >> 1) - es;
+        float ec[6], en[6], tv[8];
+#pragma unroll
+        for (int i = 0; i < 6; ++i) {
+            ec[i] = pr[i * es];
+            en[i] = pr[i * es + (odd ? 1 : -1)];
+        }
+#pragma unroll
+        for (int j = 0; j < 8; ++j) tv[j] = tc[j * ts];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            const int i = 1 + (j >> 1), m = (j & 1) ? i + 1 : i - 1;
+            const bool unk = (j < 4 ? lo2(keep[j]) : hi2(keep[j - 4])) != 0.f;
+            const float bl = prolong_blend(ec[i], ec[m], en[i], en[m]);
+            const float a = unk ? bl : 0.f;
+            tc[j * ts] = PRO == 1 ? __fadd_rn(tv[j], a) : (unk ? a : tv[j]);
+            pmax = fmaxf(pmax, fabsf(a));
+        }
+        {
+            const bool row = wrp < 2;
+            const int half = 1 + (lane >> 1), far = (wrp & 1) ? B / 2 + 1 : 0;
+            const float* pp = pw + (row ? far * EW + half : half * EW + far);
+            const int in = (row ? EW : 1) * ((wrp & 1) ? -1 : 1);
+            const int al = (row ? 1 : EW) * (odd ? 1 : -1);
+            const int vn = row ? in : al, hn = row ? al : in;
+            const float a = prolong_blend(pp[0], pp[vn], pp[hn], pp[vn + hn]);
+            float* tp = s_u + du + (row ? ((wrp & 1) ? (B + 1) * P : 0) + lane + 1
+                                        : (lane + 1) * P + ((wrp & 1) ? B + 1 : 0));
+            const float old = *tp;
+            *tp = hkn ? old : (PRO == 1 ? __fadd_rn(old, a) : a);
+        }
+        __syncthreads();  // the residual reads the other threads' columns
+    }
+
+    // residual (block_residual's sums)
+    f2 r[4];
+    {
+        float rv[8];
+        const float* bc = s_b + db + r0 * PB + lane;
+        const float dh = (float)((gx > 0) + (gx < w - 1)) + 2.f;
+        float up = 0.f, cen = 0.f;
+        if (!zero_in) {
+            up = tc[-ts];
+            cen = tc[0];
+        }
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            float v = rhs_zero ? 0.f : bc[j * dr * PB];
+            if (!zero_in) {
+                const float* c0 = tc + j * ts;
+                const float dn = c0[ts];
+                const int gy = y0 + r0 + dr * j;
+                const float e = (float)((gy == 0) + (gy == h - 1));
+                const float nb = (up + dn) + (c0[-1] + c0[1]);
+                const float a = __fmaf_rn(e - dh, cen, nb);
+                v = rhs_zero ? a : v + a;
+                up = cen;
+                cen = dn;
+            }
+            rv[j] = v;
+        }
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+            r[k] = pk(rv[k] * lo2(keep[k]), rv[k + 4] * hi2(keep[k]));
+    }
+
+    // CG (block_cg's steps); sums: the column pairs of the two-warp form's
+    // threads, the warp, then the row groups and the halves
+    auto block_sum4 = [&](f2 acc, float4* red) {
+        acc = add2(acc, __shfl_xor_sync(kFull, acc, 1));
+        float v = lo2(acc) + hi2(acc);
+#pragma unroll
+        for (int d = 16; d > 1; d >>= 1) v += __shfl_xor_sync(kFull, v, d);
+        if (lane == 0) reinterpret_cast<float*>(red)[wrp] = v;
+        __syncthreads();
+        const float4 a = *red;
+        return (a.x + a.y) + (a.z + a.w);
+    };
+    auto publish = [&]() {  // the rows that other warps need
+        if (g) s_row0[wi][lane] = lo2(r[0]);
+        s_row7[wrp][lane] = hi2(r[3]);
+    };
+    f2 x[4], p[4], q[4];
+    f2 acc = mul2(r[0], r[0]);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        p[k] = r[k];
+        x[k] = 0ull;
+        if (k) acc = fma2(r[k], r[k], acc);
+    }
+    publish();
+    float rr = block_sum4(acc, &s_red2);
+    float pb = g ? s_row0[wi ^ 1][lane] : 0.f;  // local row -1 of p
+    float p8 = s_row7[wrp ^ 1][lane];           // local row 8
+    const float rr_stop = fmaxf(rtol2 >= 0.f ? fmaxf(rtol2, 1e-14f) * rr : fmaxf(1e-14f * rr, -rtol2),
+                                FLT_MIN);
+    int it = 0;
+    while (it < iters && rr > rr_stop) {
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const f2 in = __shfl_xor_sync(kFull, p[k], 1);
+            const f2 ou = __shfl_sync(kFull, p[k], outer);
+            f2 nb;
+            if (k == 0) nb = pk(pb + lo2(p[1]), lo2(p[3]) + hi2(p[1]));
+            else if (k == 3) nb = pk(lo2(p[2]) + hi2(p[0]), hi2(p[2]) + p8);
+            else nb = add2(p[k - 1], p[k + 1]);
+            nb = add2(nb, in);
+            nb = fma2(mo2, ou, nb);
+            q[k] = mul2(fma2(nd[k], p[k], nb), keep[k]);
+            acc = k ? fma2(p[k], q[k], acc) : mul2(p[k], q[k]);
+        }
+        const float pq = -block_sum4(acc, &s_red1);
+        if (!(pq >= FLT_MIN && pq <= FLT_MAX)) break;
+        const float a = quotient(rr, pq);
+        const f2 a2 = pk(a, a);
+        if (++it == iters) {
+#pragma unroll
+            for (int k = 0; k < 4; ++k) x[k] = fma2(a2, p[k], x[k]);
+            break;
+        }
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            x[k] = fma2(a2, p[k], x[k]);
+            r[k] = fma2(a2, q[k], r[k]);
+            acc = k ? fma2(r[k], r[k], acc) : mul2(r[k], r[k]);
+        }
+        publish();
+        const float rrn = block_sum4(acc, &s_red2);
+        const float beta = quotient(rrn, rr);
+        rr = rrn;
+        const f2 b2 = pk(beta, beta);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) p[k] = fma2(b2, p[k], r[k]);
+        if (g) pb = fmaf(beta, pb, s_row0[wi ^ 1][lane]);
+        p8 = fmaf(beta, p8, s_row7[wrp ^ 1][lane]);
+    }
+
+    // the weighted write (k_oras_2w)
+    float vmax = 0.f;
+    float* const up = u_out + ch * n + (size_t)(y0 + r0) * w + gx;
+    const ptrdiff_t us = dr * (ptrdiff_t)w;
+    if constexpr (OV == 0) {
+        // local row 0 of g = 0 is the block's edge row: weight 0 inside the image
+        if (!g && (wi == 0 ? ky > 0 : ky < nby - 1)) own &= ~1u;
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            const float v = j < 4 ? lo2(x[j]) : hi2(x[j - 4]);
+            if (wx > 0.f && ((own >> j) & 1u)) {
+                up[j * us] = (zero_in ? 0.f : tc[j * ts]) + v;
+                vmax = fmaxf(vmax, fabsf(v));
+            }
+        }
+    } else {
+        const int first = shared_first(o), last = first + shared_per_seam(o);
+        const bool xf = !(kx > 0 && lane >= first && lane < last);
+        float* const mine = parked + ((size_t)blk * C + ch) * (B * B) + lane;
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            const int ly = r0 + dr * j;
+            const float d = wx * s_wy[ly];
+            const float v = j < 4 ? lo2(x[j]) : hi2(x[j - 4]);
+            const float u = zero_in ? 0.f : tc[j * ts];
+            const bool yf = !(ky > 0 && ly >= first && ly < last);
+            const float a = shared_part(d, v, u, xf && yf);
+            if (d == 1.f) up[j * us] = a;
+            else if (d > 0.f) mine[ly * B] = a;
+            if (d > 0.f) vmax = fmaxf(vmax, fabsf(v));
+        }
+    }
+    if (step_count && t == 0) atomicAdd(step_count, (unsigned long long)it);
+    if (maxupd) {
+        vmax = warp_max(vmax);
+        if (lane == 0 && vmax > 0.f) atomicMax(maxupd, __float_as_uint(vmax));
+    }
+    if (PRO == 1 && maxpro) {
+        pmax = warp_max(pmax);
+        if (lane == 0 && pmax > 0.f) atomicMax(maxpro, __float_as_uint(pmax));
+    }
+}
 
 // ---- 16-bit storage variant of k_oras_2w ------------------------------------
 // The CG vectors, the stencil and the vector updates of each local solve run
@@ -3298,6 +3661,13 @@ const void* oras_2w_h_fn() {
     return (const void*)k_oras_2w_h<H, TU, F64>;
 }
 
+// Local problems of a launch up to which the four-warp form takes it: four per
+// SM, what is resident at once at 96 registers with room for a tile more.
+// Decodes of 256x256 / 481x321 RGB / 1920x1080 RGB with the line at 0, 1, 2, 4
+// and 6 per SM: 249, 212, 212, 211, 211 / 432, 404, 396, 394, 393 / 1115, 1094,
+// 1094, 1091, 1088 us; four 4K decodes in flight 4764, 4749, 4755, 4771, 4769.
+constexpr int kQuadTasks = 152 * 4;
+
 // precision: 0 FP32 iterates (tiles by TMA where the image allows it), 1 FP16,
 // 2 BF16 iterates; stor: storage of u_in, rhs, u_out (kF32, or the iterate
 // type on the coarse levels of the 16-bit modes); f64: FP64 block residual.
@@ -3365,7 +3735,13 @@ cudaError_t launch_oras_2w(const float* u_in, int zero_in, const float* rhs, int
     int grid = chan_inner ? slots : (ntasks < slots ? ntasks : slots);
     if (grid < 1) grid = 1;
     if (ev) record_event(ev[0], s);
-    if (precision == 0) {
+    if (precision == 0 && !f64 && (o & 1) == 0 && ntasks <= kQuadTasks) {
+        auto* const fn4 = o == 2 ? (pm == 1 ? k_oras_4w<1, 0> : pm == 2 ? k_oras_4w<2, 0> : k_oras_4w<0, 0>)
+                                 : (pm == 1 ? k_oras_4w<1, 1> : pm == 2 ? k_oras_4w<2, 1> : k_oras_4w<0, 1>);
+        fn4<<<ntasks, 128, 0, s>>>(u_in, zero_in, rhs, rhs_zero, mbits, wpr, w, h, C, o, nbx, nby,
+                                   alpha, iters, rtol2, u_out, parked, maxupd, tm_u, tm_b, use_tma,
+                                   errflag, step_count, pro_e, wH, hH, pro_max, tm_e, use_tma_e);
+    } else if (precision == 0) {
         fn<<<grid, 64, smem, s>>>(u_in, zero_in, rhs, rhs_zero, mbits, wpr, w, h, C, o, nbx, nby,
                                   alpha, iters, rtol2, u_out, parked, maxupd, chan_inner, tm_u,
                                   tm_b, use_tma, errflag, step_count, pro_e, wH, hH, pro_max,

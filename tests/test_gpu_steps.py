@@ -288,6 +288,98 @@ def test_oras_block_edges(di, h, w, o):
                               out)
 
 
+QUAD_CASES = [  # (h, w, overlap, aligned): up to 608 local problems in one channel, more in four
+    (601, 600, 2, True), (500, 601, 6, True), (601, 640, 4, False), (660, 580, 2, False),
+]
+
+
+@pytest.mark.parametrize("h,w,o,aligned", QUAD_CASES)
+@pytest.mark.parametrize("rhs_zero", [True, False])
+def test_oras_few_problems_same_bits(di, h, w, o, aligned, rhs_zero):
+    # launches of few local problems take four warps per problem, larger ones two:
+    # one channel alone and the same channel among four give the same bits, for
+    # the plain iteration and both prolonged starts
+    f, fn, c = _case(h, w, 1, 0.06, h + 3 * w + o)
+    g = np.random.default_rng(w)
+    H, W = M.coarse_shape(h, w)
+    known = c.astype(bool)
+    if rhs_zero:
+        u = np.where(known, f, g.uniform(0, 255, f.shape)).astype(np.float32)
+        b = fn
+    else:
+        u = np.where(known, 0.0, g.normal(size=f.shape)).astype(np.float32)
+        b = np.where(known, 0.0, g.normal(size=f.shape)).astype(np.float32)
+    uH = g.uniform(0, 255, size=(1, H, W)).astype(np.float32)
+    put = T if aligned else _unaligned
+    outs = []
+    with di.Context(block=32, overlap=o, alpha=0.3) as ctx:
+        for C in (1, 4):
+            ub, bb, eb = (np.repeat(a, C, axis=0) for a in (u, b, uH))
+            r = [ctx.oras_iteration(put(ub), put(bb), T(c), 7, rhs_zero=rhs_zero),
+                 ctx.prolong_oras_iteration(T(eb), put(ub), put(bb), T(c), 7, rhs_zero=rhs_zero),
+                 ctx.oras_iteration(put(ub), put(bb), T(c), 400, rhs_zero=rhs_zero)]
+            if rhs_zero:
+                r.append(ctx.prolong_oras_iteration(T(eb), put(bb), put(bb), T(c), 7, rhs_zero=True,
+                                                    mode=0))
+            outs.append([N(x) for x in r])
+    for a, b4 in zip(*outs):
+        assert np.isfinite(a).all()
+        for ch in range(4):
+            assert np.array_equal(a[0], b4[ch])
+
+
+@pytest.mark.parametrize("w", [16, 48, 64, 112, 4112])
+@pytest.mark.parametrize("h", [1, 31, 33, 130])
+def test_packed_mask_sixteen_columns_at_a_time(di, h, w):
+    # rows of whole 16-byte groups: the unknown count and the solution's mask
+    # pixels show the packed words
+    f, fn, c = _case(h, w, 1, 0.1, 5 * h + w)
+    c[-1, -1] = 1
+    fn[:, -1, -1] = f[:, -1, -1]
+    with di.Context(max_cycles=2, stop_rule=2) as ctx:
+        u, _ = ctx.inpaint(T(fn), T(c))
+        assert ctx.stats()["unknowns"] == int((c == 0).sum())
+    assert np.array_equal(N(u)[:, c == 1], f[:, c == 1])
+    g = np.random.default_rng(3)
+    u0 = np.where(c.astype(bool), f, g.uniform(0, 255, f.shape)).astype(np.float32)
+    with di.Context(block=32, overlap=2) as ctx:  # the same mask off the 16-byte boundary
+        flat = torch.empty(c.size + 1, dtype=torch.uint8, device=DEV)
+        co = flat[1:].view(c.shape)
+        co.copy_(torch.from_numpy(c))
+        a = N(ctx.oras_iteration(T(u0), T(fn), T(c), 5, rhs_zero=True))
+        assert np.array_equal(N(ctx.oras_iteration(T(u0), T(fn), co, 5, rhs_zero=True)), a)
+
+
+@pytest.mark.parametrize("h,w", [(1999, 2003), (1201, 2048), (577, 3333)])
+def test_pyramid_level_large_and_odd(di, h, w):
+    # four rows of cells per thread: the same bits as the separate steps at
+    # ragged rows and columns
+    f, fn, c = _case(h, w, 3, 0.05, h + w)
+    cH, bH, _, unk = di.pyramid_level(T(c), T(fn))
+    cH_ref = M.mask_downsample(c)
+    assert np.array_equal(N(cH), cH_ref) and int(N(unk)[0]) == int((cH_ref == 0).sum())
+    assert np.array_equal(N(bH), N(di.values_downsample(T(c), T(fn), T(cH_ref))))
+
+
+@pytest.mark.parametrize("C", [2, 3, 4])
+@pytest.mark.parametrize("h,w,aligned", [(1200, 1100, True), (1101, 1203, True), (1200, 1100, False)])
+@pytest.mark.parametrize("rhs_zero", [True, False])
+def test_restrict_all_channels_of_a_cell(di, h, w, C, aligned, rhs_zero):
+    # large levels restrict every channel of a cell in one thread: the same bits
+    # as channel by channel
+    f, fn, c = _case(h, w, C, 0.05, h + C)
+    g = np.random.default_rng(C)
+    u = np.where(c.astype(bool), f, g.uniform(0, 255, f.shape)).astype(np.float32)
+    b = fn if rhs_zero else g.normal(size=f.shape).astype(np.float32)
+    put = T if aligned else _unaligned
+    cH = di.mask_downsample(T(c))
+    r = N(di.restrict_residual(put(u), put(b), T(c), cH, rhs_zero=rhs_zero))
+    for ch in range(C):
+        one = N(di.restrict_residual(put(u[ch:ch + 1]), put(b[ch:ch + 1]), T(c), cH,
+                                     rhs_zero=rhs_zero))
+        assert np.array_equal(r[ch], one[0])
+
+
 PRO_CASES = [  # (h, w, overlap, rhs_zero, aligned)
     (70, 96, 2, True, True), (70, 96, 2, False, False), (70, 96, 6, False, True),
     (33, 35, 2, False, True), (130, 100, 2, True, False), (61, 250, 6, True, True),
