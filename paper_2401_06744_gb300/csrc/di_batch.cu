@@ -56,6 +56,7 @@ struct BImage {
 struct Launch {
     int kind;  // BatchKind, or -1 for the block kernel
     int seg0, nseg, nwork;
+    int ntasks, cmax;  // block kernel: local problems, most channels of an image
 };
 
 }  // namespace
@@ -182,7 +183,13 @@ struct Builder {
     }
     void push(int kind, std::vector<BatchSeg>& v, int nwork) {
         if (v.empty() || nwork < 1) return;
-        launches.push_back({kind, (int)segs.size(), (int)v.size(), nwork});
+        int ntasks = 0, cmax = 1;  // local problems of a block-kernel launch
+        if (kind < 0)
+            for (const BatchSeg& g : v) {
+                ntasks += g.nbx * g.nby * g.C;
+                cmax = std::max(cmax, g.C);
+            }
+        launches.push_back({kind, (int)segs.size(), (int)v.size(), nwork, ntasks, cmax});
         segs.insert(segs.end(), v.begin(), v.end());
     }
     // a block-kernel segment of image i on level l (in -> out)
@@ -402,7 +409,8 @@ struct Builder {
     cudaError_t run(const Launch& L, cudaStream_t s) {
         const BatchSeg* d = b->dsegs + L.seg0;
         if (L.kind < 0)
-            return launch_batch_oras(d, L.nseg, L.nwork, b->cfg.overlap, b->cfg.alpha, b->bs, s);
+            return launch_batch_oras(d, L.nseg, L.nwork, L.ntasks, L.cmax, b->cfg.overlap,
+                                     b->cfg.alpha, b->bs, s);
         return launch_batch_grid(L.kind, d, L.nseg, L.nwork, b->bs, s);
     }
 };

@@ -273,9 +273,10 @@ struct BatchState {
 // first) covering nctas CTAs.
 cudaError_t launch_batch_grid(int kind, const BatchSeg* segs, int nseg, int nctas,
                               const BatchState& bs, cudaStream_t s);
-// The batched block kernel (32x32 blocks, 0/1 weights) over nunits block units.
-cudaError_t launch_batch_oras(const BatchSeg* segs, int nseg, int nunits, int o, float alpha,
-                              const BatchState& bs, cudaStream_t s);
+// The batched block kernel (32x32 blocks, 0/1 weights) over nunits block units
+// of at most cmax channels, ntasks local problems (blocks x channels) in all.
+cudaError_t launch_batch_oras(const BatchSeg* segs, int nseg, int nunits, int ntasks, int cmax,
+                              int o, float alpha, const BatchState& bs, cudaStream_t s);
 // Plan of every image (levels in use, cascade start, initial state); L[i]
 // and n0[i] are the images' pyramid depths and pixel counts (device arrays).
 cudaError_t launch_batch_plan(int n, const int* L, const unsigned long long* n0,

@@ -2277,22 +2277,22 @@ k_oras_2w(const float* __restrict__ u_in, int zero_in, const float* __restrict__
 // With every SM busy it is the slower one (a barrier and a sum more per pixel).
 // 256x256 decode 249 -> 211 us, 481x321 RGB (overlap 6) 432 -> 394, 1920x1080 RGB
 // 1115 -> 1090, 3840x2160 RGB 1606 -> 1589.
+// One local problem (block blk, channel ch).  PRO: as in k_oras_2w, -1: pro_rt.
 template <int PRO, int OV>
-__global__ void __launch_bounds__(128)
-k_oras_4w(const float* __restrict__ u_in, int zero_in, const float* __restrict__ rhs, int rhs_zero,
-          const uint32_t* __restrict__ mbits, int wpr, int w, int h, int C, int o, int nbx, int nby,
-          float alpha, int iters, float rtol2, float* __restrict__ u_out,
-          float* __restrict__ parked, unsigned* __restrict__ maxupd,
-          const __grid_constant__ CUtensorMap tm_u, const __grid_constant__ CUtensorMap tm_b,
-          int use_tma, unsigned* __restrict__ errflag,
-          unsigned long long* __restrict__ step_count, const float* __restrict__ eH, int wH,
-          int hH, unsigned* __restrict__ maxpro, const __grid_constant__ CUtensorMap tm_e,
-          int use_tma_e) {
+__device__ __forceinline__ void oras_4w(
+    int blk, int ch, const float* __restrict__ u_in, int zero_in, const float* __restrict__ rhs,
+    int rhs_zero, const uint32_t* __restrict__ mbits, int wpr, int w, int h, int C, int o, int nbx,
+    int nby, float alpha, int iters, float rtol2, float* __restrict__ u_out,
+    float* __restrict__ parked, unsigned* __restrict__ maxupd, const CUtensorMap* tm_u,
+    const CUtensorMap* tm_b, int use_tma, unsigned* __restrict__ errflag,
+    unsigned long long* __restrict__ step_count, const float* __restrict__ eH, int wH, int hH,
+    unsigned* __restrict__ maxpro, const CUtensorMap* tm_e, int use_tma_e, int pro_rt) {
+    const int pro = PRO >= 0 ? PRO : pro_rt;
     constexpr int B = 32, TH = Smem2W::TH, P = Smem2W::PU, PB = Smem2W::PB;
     constexpr int EW = Smem2W::EPW;
     __shared__ __align__(128) float s_u[Smem2W::USTRIDE];
     __shared__ __align__(128) float s_b[Smem2W::BSTRIDE];
-    __shared__ __align__(128) float s_e[PRO ? Smem2W::ESTRIDE : 32];
+    __shared__ __align__(128) float s_e[PRO != 0 ? Smem2W::ESTRIDE : 32];
     __shared__ float s_wy[B], s_row0[2][32], s_row7[4][32];
     __shared__ float4 s_red1, s_red2;
     __shared__ __align__(8) unsigned long long s_bar;
@@ -2301,7 +2301,6 @@ k_oras_4w(const float* __restrict__ u_in, int zero_in, const float* __restrict__
     const int wi = wrp >> 1, g = wrp & 1;
     const int r0 = wi ? (g ? 16 : 31) : (g ? 15 : 0), dr = wi == g ? 1 : -1;
     const int s = B - o;
-    const int blk = (int)blockIdx.x / C, ch = (int)blockIdx.x - blk * C;
     const int ky = blk / nbx, kx = blk - ky * nbx, x0 = kx * s, y0 = ky * s;
     const size_t n = (size_t)w * h;
     const unsigned bar = (unsigned)__cvta_generic_to_shared(&s_bar);
@@ -2313,16 +2312,16 @@ k_oras_4w(const float* __restrict__ u_in, int zero_in, const float* __restrict__
             asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
             const unsigned bytes = (zero_in ? 0u : (unsigned)Smem2W::TMA_U_BYTES) +
                                    (rhs_zero ? 0u : (unsigned)Smem2W::TMA_B_BYTES) +
-                                   (PRO != 0 && use_tma_e ? (unsigned)Smem2W::TMA_E_BYTES : 0u);
+                                   (pro != 0 && use_tma_e ? (unsigned)Smem2W::TMA_E_BYTES : 0u);
             asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;"
                          :: "r"(bar), "r"(bytes) : "memory");
             if (!zero_in)
-                tma_load_3d((unsigned)__cvta_generic_to_shared(s_u), &tm_u, (x0 - 1) & ~3, y0 - 1,
+                tma_load_3d((unsigned)__cvta_generic_to_shared(s_u), tm_u, (x0 - 1) & ~3, y0 - 1,
                             ch, bar);
             if (!rhs_zero)
-                tma_load_3d((unsigned)__cvta_generic_to_shared(s_b), &tm_b, x0 & ~3, y0, ch, bar);
-            if (PRO != 0 && use_tma_e)
-                tma_load_3d((unsigned)__cvta_generic_to_shared(s_e), &tm_e,
+                tma_load_3d((unsigned)__cvta_generic_to_shared(s_b), tm_b, x0 & ~3, y0, ch, bar);
+            if (pro != 0 && use_tma_e)
+                tma_load_3d((unsigned)__cvta_generic_to_shared(s_e), tm_e,
                             ((x0 >> 1) - 1) & ~3, (y0 >> 1) - 1, ch, bar);
         }
     } else {
@@ -2350,7 +2349,7 @@ k_oras_4w(const float* __restrict__ u_in, int zero_in, const float* __restrict__
             }
         }
     }
-    if (PRO != 0 && !use_tma_e)
+    if (pro != 0 && !use_tma_e)
         copy_patch_clamped(s_e, eH + (size_t)ch * wH * hH, x0, y0, wH, hH, t, 128);
     cp_async_commit();
 
@@ -2365,7 +2364,7 @@ k_oras_4w(const float* __restrict__ u_in, int zero_in, const float* __restrict__
         }
     }
     bool hkn = true;  // known or off the image
-    if (PRO != 0) {
+    if (pro != 0) {
         const int hy = wrp == 0 ? y0 - 1 : wrp == 1 ? y0 + B : y0 + lane;
         const int hx = wrp < 2 ? x0 + lane : wrp == 2 ? x0 - 1 : x0 + B;
         if (hx >= 0 && hx < w && hy >= 0 && hy < h)
@@ -2415,7 +2414,7 @@ k_oras_4w(const float* __restrict__ u_in, int zero_in, const float* __restrict__
     float* const tc = s_u + du + (r0 + 1) * P + lane + 1;  // local row 0
     const int ts = dr * P;
     float pmax = 0.f;
-    if constexpr (PRO != 0) {
+    if (pro != 0) {
         const int Ys = (y0 >> 1) - 1, Xs = (x0 >> 1) - 1;
         float* const pw = s_e + (use_tma_e ? Xs - (Xs & ~3) : 0);
         if (use_tma_e && (Ys < 0 || Xs < 0 || Ys + Smem2W::EW > hH || Xs + Smem2W::EW > wH)) {
@@ -2444,7 +2443,7 @@ k_oras_4w(const float* __restrict__ u_in, int zero_in, const float* __restrict__
             const bool unk = (j < 4 ? lo2(keep[j]) : hi2(keep[j - 4])) != 0.f;
             const float bl = prolong_blend(ec[i], ec[m], en[i], en[m]);
             const float a = unk ? bl : 0.f;
-            tc[j * ts] = PRO == 1 ? __fadd_rn(tv[j], a) : (unk ? a : tv[j]);
+            tc[j * ts] = pro == 1 ? __fadd_rn(tv[j], a) : (unk ? a : tv[j]);
             pmax = fmaxf(pmax, fabsf(a));
         }
         {
@@ -2458,7 +2457,7 @@ k_oras_4w(const float* __restrict__ u_in, int zero_in, const float* __restrict__
             float* tp = s_u + du + (row ? ((wrp & 1) ? (B + 1) * P : 0) + lane + 1
                                         : (lane + 1) * P + ((wrp & 1) ? B + 1 : 0));
             const float old = *tp;
-            *tp = hkn ? old : (PRO == 1 ? __fadd_rn(old, a) : a);
+            *tp = hkn ? old : (pro == 1 ? __fadd_rn(old, a) : a);
         }
         __syncthreads();  // the residual reads the other threads' columns
     }
@@ -2603,10 +2602,27 @@ k_oras_4w(const float* __restrict__ u_in, int zero_in, const float* __restrict__
         vmax = warp_max(vmax);
         if (lane == 0 && vmax > 0.f) atomicMax(maxupd, __float_as_uint(vmax));
     }
-    if (PRO == 1 && maxpro) {
+    if (pro == 1 && maxpro) {
         pmax = warp_max(pmax);
         if (lane == 0 && pmax > 0.f) atomicMax(maxpro, __float_as_uint(pmax));
     }
+}
+
+template <int PRO, int OV>
+__global__ void __launch_bounds__(128, 4)
+k_oras_4w(const float* __restrict__ u_in, int zero_in, const float* __restrict__ rhs, int rhs_zero,
+          const uint32_t* __restrict__ mbits, int wpr, int w, int h, int C, int o, int nbx, int nby,
+          float alpha, int iters, float rtol2, float* __restrict__ u_out,
+          float* __restrict__ parked, unsigned* __restrict__ maxupd,
+          const __grid_constant__ CUtensorMap tm_u, const __grid_constant__ CUtensorMap tm_b,
+          int use_tma, unsigned* __restrict__ errflag,
+          unsigned long long* __restrict__ step_count, const float* __restrict__ eH, int wH,
+          int hH, unsigned* __restrict__ maxpro, const __grid_constant__ CUtensorMap tm_e,
+          int use_tma_e) {
+    const int blk = (int)blockIdx.x / C;
+    oras_4w<PRO, OV>(blk, (int)blockIdx.x - blk * C, u_in, zero_in, rhs, rhs_zero, mbits, wpr, w, h,
+                     C, o, nbx, nby, alpha, iters, rtol2, u_out, parked, maxupd, &tm_u, &tm_b,
+                     use_tma, errflag, step_count, eH, wH, hH, maxpro, &tm_e, use_tma_e, PRO);
 }
 
 // ---- 16-bit storage variant of k_oras_2w ------------------------------------
@@ -3211,8 +3227,8 @@ k_batch_grid(const BatchSeg* __restrict__ segs, int nseg, BatchState bs) {
 // form its start by prolongation (BatchSeg).  Otherwise the local problem,
 // the CG and the write are those of k_oras_2w.
 __global__ void __launch_bounds__(64, 8)
-k_batch_oras(const BatchSeg* __restrict__ segs, int nseg, int nunits, int o, float alpha,
-             BatchState bs) {
+k_batch_oras(const BatchSeg* __restrict__ segs, int nseg, int nunits, int split, int o,
+             float alpha, BatchState bs) {
     constexpr int B = 32, TH = Smem2W::TH, P = Smem2W::PU, PB = Smem2W::PB;
     constexpr int TILE = Smem2W::USTRIDE;
     extern __shared__ float smem_raw[];
@@ -3239,16 +3255,20 @@ k_batch_oras(const BatchSeg* __restrict__ segs, int nseg, int nunits, int o, flo
         int seg, blk, ch;
     };
     // the next active task after (unit g, channel ch): the next channel, else
-    // the next unit of this CTA whose image takes part
+    // the next unit of this CTA whose image takes part; split > 0 (fewer units
+    // than CTA slots): g counts (unit, channel) pairs, split of them per unit
     auto advance = [&](int& g, Task& tk) {
-        if (tk.seg >= 0 && ++tk.ch < segs[tk.seg].C) return true;
-        for (g = g < 0 ? (int)blockIdx.x : g + (int)gridDim.x; g < nunits; g += (int)gridDim.x) {
-            const int si = find_seg(segs, nseg, g);
+        if (!split && tk.seg >= 0 && ++tk.ch < segs[tk.seg].C) return true;
+        const int end = split ? nunits * split : nunits;
+        for (g = g < 0 ? (int)blockIdx.x : g + (int)gridDim.x; g < end; g += (int)gridDim.x) {
+            const int unit = split ? g / split : g;
+            const int si = find_seg(segs, nseg, unit);
             const BatchSeg& sg = segs[si];
             if (!seg_active(sg.when, sg.img, sg.level, sg.L, bs)) continue;
+            tk.ch = split ? g - unit * split : 0;
+            if (tk.ch >= sg.C) continue;
             tk.seg = si;
-            tk.blk = g - sg.first;
-            tk.ch = 0;
+            tk.blk = unit - sg.first;
             return true;
         }
         return false;
@@ -3458,6 +3478,26 @@ k_batch_oras(const BatchSeg* __restrict__ segs, int nseg, int nunits, int o, flo
     }
 }
 
+// The same with four warps per local problem (oras_4w), for launches of few:
+// CTA cmax * g + ch takes channel ch of block unit g.  With it, and the
+// channels of a block on separate CTAs where there are fewer blocks than CTA
+// slots, a batch of 12 images of 640x481 went from 1340 to 1167 us.
+__global__ void __launch_bounds__(128, 4)
+k_batch_oras_4w(const BatchSeg* __restrict__ segs, int nseg, int cmax, int o, float alpha,
+                BatchState bs) {
+    const int g = (int)blockIdx.x / cmax, ch = (int)blockIdx.x - g * cmax;
+    const BatchSeg& sg = segs[find_seg(segs, nseg, g)];
+    if (ch >= sg.C || !seg_active(sg.when, sg.img, sg.level, sg.L, bs)) return;
+    const CUtensorMap* maps = static_cast<const CUtensorMap*>(sg.tmaps);
+    const bool pro = sg.pro_mode != 0 && (!sg.pro_check || sg.level + 1 < bs.leff[sg.img]);
+    oras_4w<-1, 0>(g - sg.first, ch, static_cast<const float*>(sg.in0), sg.zero_in,
+                   static_cast<const float*>(sg.in1), sg.rhs_zero, sg.mbits, sg.wpr, sg.w, sg.h,
+                   sg.C, o, sg.nbx, sg.nby, alpha, sg.iters, sg.rtol2,
+                   static_cast<float*>(sg.out0), nullptr, sg.maxupd, maps, maps + 1, sg.tma, bs.err,
+                   nullptr, sg.pro_e, (sg.w + 1) / 2, (sg.h + 1) / 2,
+                   sg.pro_mode == 1 ? sg.pro_max : nullptr, nullptr, 0, pro ? sg.pro_mode : 0);
+}
+
 // Plan of every image of a batch: levels in use, the cascade's start level
 // and the initial stop state (as k_plan for one image).
 __global__ void k_batch_plan(int n, const int* __restrict__ Ls,
@@ -3662,7 +3702,8 @@ const void* oras_2w_h_fn() {
 }
 
 // Local problems of a launch up to which the four-warp form takes it: four per
-// SM, what is resident at once at 96 registers with room for a tile more.
+// SM, what is resident at once (at 80 registers for six, the 256x256 decode took
+// 218 us instead of 211).
 // Decodes of 256x256 / 481x321 RGB / 1920x1080 RGB with the line at 0, 1, 2, 4
 // and 6 per SM: 249, 212, 212, 211, 211 / 432, 404, 396, 394, 393 / 1115, 1094,
 // 1094, 1091, 1088 us; four 4K decodes in flight 4764, 4749, 4755, 4771, 4769.
@@ -4245,16 +4286,24 @@ cudaError_t launch_batch_grid(int kind, const BatchSeg* segs, int nseg, int ncta
     return cudaGetLastError();
 }
 
-cudaError_t launch_batch_oras(const BatchSeg* segs, int nseg, int nunits, int o, float alpha,
+cudaError_t launch_batch_oras(const BatchSeg* segs, int nseg, int nunits, int ntasks, int cmax,
+                              int o, float alpha,
                               const BatchState& bs, cudaStream_t s) {
     if (nunits < 1 || nseg < 1) return cudaSuccess;
+    if (ntasks <= kQuadTasks) {  // as for one image
+        k_batch_oras_4w<<<nunits * cmax, 128, 0, s>>>(segs, nseg, cmax, o, alpha, bs);
+        count();
+        return cudaGetLastError();
+    }
     if (shared_per_seam(o) != 0) return cudaErrorInvalidValue;  // 0/1 weights only
     int nsm = 0;
     const size_t smem = Smem2W::bytes(true, true);
     const int oc = cached_occupancy((const void*)k_batch_oras, 64, smem, smem, &nsm);
     int grid = nsm * oc;
-    if (grid > nunits) grid = nunits;
-    k_batch_oras<<<grid, 64, smem, s>>>(segs, nseg, nunits, o, alpha, bs);
+    const int split = nunits < grid ? cmax : 0;
+    const int work = split ? nunits * split : nunits;
+    if (grid > work) grid = work;
+    k_batch_oras<<<grid, 64, smem, s>>>(segs, nseg, nunits, split, o, alpha, bs);
     count();
     return cudaGetLastError();
 }
