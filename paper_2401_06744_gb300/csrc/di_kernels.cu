@@ -2662,7 +2662,7 @@ struct Bf16T {
 // the coarse levels in the 16-bit precision modes (tiles read and widened to
 // FP32 at the start of each task).  F64: the block residual in FP64.
 template <class H, class TU, bool F64>
-__global__ void __launch_bounds__(64, 10)
+__global__ void __launch_bounds__(64, 8)
 k_oras_2w_h(const TU* __restrict__ u_in, int zero_in, const TU* __restrict__ rhs,
             int rhs_zero, const uint32_t* __restrict__ mbits, int wpr, int w, int h, int C, int o,
             int nbx, int nby, float alpha, int iters, float rtol2, TU* __restrict__ u_out,
@@ -2702,48 +2702,73 @@ k_oras_2w_h(const TU* __restrict__ u_in, int zero_in, const TU* __restrict__ rhs
     // loads widened to FP32 (16-bit storage)
     auto tiles = [&](int blk, int ch, int bs) {
         const int px0 = (blk % nbx) * s, py0 = (blk / nbx) * s;
-        if (!zero_in) {
-            const TU* src = u_in + ch * n;
-            float* dst = s_u + bs * TILE;
-            const int gxa = px0 - 1 + lane, gxb = gxa + 32;
-            const bool oka = gxa >= 0 && gxa < w;
-            const bool okb = lane < TH - 32 && gxb < w;
+        if (kAsync) {
+            if (!zero_in) {
+                const float* src = reinterpret_cast<const float*>(u_in + ch * n);
+                float* dst = s_u + bs * TILE;
+                const int gxa = px0 - 1 + lane, gxb = gxa + 32;
+                const bool oka = gxa >= 0 && gxa < w;
+                const bool okb = lane < TH - 32 && gxb < w;
 #pragma unroll 2
-            for (int ty = wi; ty < TH; ty += 2) {
-                const int gy = py0 - 1 + ty;
-                const bool rok = gy >= 0 && gy < h;
-                const TU* row = src + (ptrdiff_t)gy * w;
-                if (kAsync) {
-                    cp_async4(dst + ty * P + lane,
-                              reinterpret_cast<const float*>((rok && oka) ? row + gxa : src),
-                              rok && oka);
+                for (int ty = wi; ty < TH; ty += 2) {
+                    const int gy = py0 - 1 + ty;
+                    const bool rok = gy >= 0 && gy < h;
+                    const float* row = src + (ptrdiff_t)gy * w;
+                    cp_async4(dst + ty * P + lane, (rok && oka) ? row + gxa : src, rok && oka);
                     if (lane < TH - 32)
-                        cp_async4(dst + ty * P + lane + 32,
-                                  reinterpret_cast<const float*>((rok && okb) ? row + gxb : src),
+                        cp_async4(dst + ty * P + lane + 32, (rok && okb) ? row + gxb : src,
                                   rok && okb);
-                } else {
-                    dst[ty * P + lane] = (rok && oka) ? ldf(row + gxa) : 0.f;
-                    if (lane < TH - 32) dst[ty * P + lane + 32] = (rok && okb) ? ldf(row + gxb) : 0.f;
                 }
+            }
+            if (!rhs_zero) {
+                const float* src = reinterpret_cast<const float*>(rhs + ch * n);
+                float* dst = s_b + bs * B * B;
+                const int gx = px0 + lane;
+#pragma unroll 4
+                for (int ly = wi; ly < B; ly += 2) {
+                    const int gy = py0 + ly;
+                    const bool ok = gx < w && gy < h;
+                    cp_async4(dst + ly * B + lane, ok ? src + (size_t)gy * w + gx : src, ok);
+                }
+            }
+            cp_async_commit();
+            return;
+        }
+        // 16-bit storage: every load of the thread (its rows of both tiles)
+        // before the first store, so that they wait together; two rows at a time
+        // the tiles took 7 us of a small level's launch
+        constexpr int NR = TH / 2, NB = B / 2;
+        float ra[NR], rb[NR], vb[NB];
+        const TU* su = u_in + ch * n;
+        const TU* sb = rhs + ch * n;
+        const int gxa = px0 - 1 + lane, gxb = gxa + 32, gx = px0 + lane;
+        const bool oka = !zero_in && gxa >= 0 && gxa < w;
+        const bool okb = !zero_in && lane < TH - 32 && gxb < w;
+#pragma unroll
+        for (int i = 0; i < NR; ++i) {
+            const int gy = py0 - 1 + wi + 2 * i;
+            const bool rok = gy >= 0 && gy < h;
+            ra[i] = rok && oka ? ldf(su + (ptrdiff_t)gy * w + gxa) : 0.f;
+            rb[i] = rok && okb ? ldf(su + (ptrdiff_t)gy * w + gxb) : 0.f;
+        }
+#pragma unroll
+        for (int i = 0; i < NB; ++i) {
+            const int gy = py0 + wi + 2 * i;
+            vb[i] = !rhs_zero && gx < w && gy < h ? ldf(sb + (size_t)gy * w + gx) : 0.f;
+        }
+        if (!zero_in) {
+            float* dst = s_u + bs * TILE + wi * P;
+#pragma unroll
+            for (int i = 0; i < NR; ++i) {
+                dst[2 * i * P + lane] = ra[i];
+                if (lane < TH - 32) dst[2 * i * P + lane + 32] = rb[i];
             }
         }
         if (!rhs_zero) {
-            const TU* src = rhs + ch * n;
-            float* dst = s_b + bs * B * B;
-            const int gx = px0 + lane;
-#pragma unroll 4
-            for (int ly = wi; ly < B; ly += 2) {
-                const int gy = py0 + ly;
-                const bool ok = gx < w && gy < h;
-                if (kAsync)
-                    cp_async4(dst + ly * B + lane,
-                              reinterpret_cast<const float*>(ok ? src + (size_t)gy * w + gx : src),
-                              ok);
-                else
-                    dst[ly * B + lane] = ok ? ldf(src + (size_t)gy * w + gx) : 0.f;
-            }
+            float* dst = s_b + bs * B * B + wi * B;
+#pragma unroll
+            for (int i = 0; i < NB; ++i) dst[2 * i * B + lane] = vb[i];
         }
-        if (kAsync) cp_async_commit();
     };
     auto prefetch = [&](int blk, int ch, int bs, int have_blk) {
         const int px0 = (blk % nbx) * s, py0 = (blk / nbx) * s;
@@ -2872,8 +2897,9 @@ k_oras_2w_h(const TU* __restrict__ u_in, int zero_in, const TU* __restrict__ rhs
         // rtol2 >= 0: relative stop (r.r <= max(rtol2, 1e-14) (r.r)_0); rtol2 < 0:
         // also stop once r.r <= -rtol2 (an absolute level, or the FP32 floor). rr is
         // the normalised residual's, so the absolute level is scaled by isc^2 too.
-        const float rr_stop = rtol2 >= 0.f ? fmaxf(rtol2, 1e-14f) * rr
-                                           : fmaxf(1e-14f * rr, -rtol2 * isc * isc);
+        const float rr_stop = fmaxf(rtol2 >= 0.f ? fmaxf(rtol2, 1e-14f) * rr
+                                                 : fmaxf(1e-14f * rr, -rtol2 * isc * isc),
+                                    FLT_MIN);
         bool bad = !(rr < INFINITY);
 
         for (int it = 0; it < iters; ++it) {
@@ -2901,11 +2927,11 @@ k_oras_2w_h(const TU* __restrict__ u_in, int zero_in, const TU* __restrict__ rhs
             if (lane == 0) s_red1[wi] = part;
             __syncthreads();
             const float pq = -(s_red1[0] + s_red1[1]);
-            if (!(pq > 0.f) || !(pq < INFINITY)) {
+            if (!(pq >= FLT_MIN) || !(pq < INFINITY)) {
                 bad = !(pq < INFINITY) || pq != pq;
                 break;
             }
-            const float a = __fdividef(rr, pq);
+            const float a = quotient(rr, pq);
             const T2 a2 = H::make(a, a);
             acc0 = 0ull;
             acc1 = 0ull;
@@ -2924,7 +2950,7 @@ k_oras_2w_h(const TU* __restrict__ u_in, int zero_in, const TU* __restrict__ rhs
             __syncthreads();
             const float rrn = s_red2[0] + s_red2[1];
             if (!(rrn < INFINITY)) { bad = true; break; }
-            const float beta = __fdividef(rrn, rr);
+            const float beta = quotient(rrn, rr);
             rr = rrn;
             const T2 b2 = H::make(beta, beta);
 #pragma unroll
