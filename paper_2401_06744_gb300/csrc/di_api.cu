@@ -72,8 +72,8 @@ struct di_ctx {
     double* partials = nullptr;     // residual norm partial sums
     size_t partials_cap = 0;
     double* norm2 = nullptr;        // [kMaxChannels]
-    unsigned long long* counts = nullptr;  // [kMaxLevels + 1]
-    unsigned* upd = nullptr;        // [kMaxUpdSlots] per-cycle max update (float bits)
+    unsigned long long* counts = nullptr;  // [kMaxLevels + 1], then upd's words
+    unsigned* upd = nullptr;        // [kMaxUpdSlots + 1] per-cycle max update (float bits), flag
     void* host = nullptr;           // pinned staging for small device->host reads
     Level lv[kMaxLevels];
     int L = 0;
@@ -103,7 +103,7 @@ struct di_ctx {
     long long g_oras = 0, g_pxch = 0, g_tasks = 0, g_pro = 0;  // profile counters of one replay
     unsigned long long* dsteps = nullptr;  // device: completed finest-level local CG steps
     // device-driven decode (see DecodeGraph): stop-test state on the device,
-    // its pinned host copy, the capture streams of the graph and its bodies,
+    // its pinned host copy (written by the device), the capture streams of the graph and its bodies,
     // and a cache of whole-decode graphs keyed by the call's buffers
     StopState* dstate = nullptr;
     StopState* hstate = nullptr;
@@ -740,9 +740,7 @@ bool capture_decode(di_ctx* ctx, Sched& S, const float* f, const uint8_t* c, flo
         auto run = [&]() -> bool {
             // 1. pyramids with the unknown counts, then the plan
             step = "pyramid";
-            if (cudaMemsetAsync(cnt, 0, (kMaxLevels + 1) * sizeof(unsigned long long), s0) ||
-                cudaMemsetAsync(ctx->upd, 0, (kMaxUpdSlots + 1) * sizeof(unsigned), s0))
-                return false;
+            if (cudaMemsetAsync(cnt, 0, kCountBytes + kUpdBytes, s0)) return false;
             if (launch_pack_mask(c, w, h, lv[0].mbits, cnt + 1, s0)) return false;
             for (int l = 1; l < L; ++l) {
                 Level& fl = lv[l - 1];
@@ -752,7 +750,7 @@ bool capture_decode(di_ctx* ctx, Sched& S, const float* f, const uint8_t* c, flo
                                          cascade ? 1 : 0, cl.mbits, cnt + 1 + l, s0))
                     return false;
             }
-            if (launch_plan(cnt, ctx->dstate, pp, s0)) return false;
+            if (launch_plan(cnt, ctx->dstate, ctx->hstate, pp, s0)) return false;
             // 2. the given start, and the reference norm of the relative-residual rule
             if (!cascade && launch_select(f, c, w, h, C, u, s0, 1)) return false;
             step = "reference norm";
@@ -793,7 +791,8 @@ bool capture_decode(di_ctx* ctx, Sched& S, const float* f, const uint8_t* c, flo
                              launch_reduce_partials(ctx->partials, nparts, C,
                                                     state_field(ctx, kNorm2), s2)))
                             return false;
-                        return launch_stop(ctx->upd, ctx->dstate, sp, pp.h_loop[v], s2) ==
+                        return launch_stop(ctx->upd, ctx->dstate, ctx->hstate, sp, pp.h_loop[v],
+                                           s2) ==
                                cudaSuccess;
                     });
                     S.s = s1;
@@ -917,8 +916,6 @@ bool device_decode(di_ctx* ctx, Sched& S, const float* f, const uint8_t* c, floa
     hit->used = ++ctx->graph_clock;
     cudaStream_t s = S.s;
     cudaError_t e = cudaGraphLaunch(hit->exec, s);
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync(ctx->hstate, ctx->dstate, sizeof(StopState), cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaEventRecord(ctx->done_ev, s);
     if (e != cudaSuccess) {
         *st = cuda_fail(ctx, e, "device-driven decode");
@@ -990,10 +987,11 @@ di_status di_create(const di_config* cfg, int device, di_ctx** out) {
     ctx->err[0] = 0;
     cudaError_t e = cudaSetDevice(device);
     if (e == cudaSuccess) e = cudaMalloc(&ctx->norm2, kMaxChannels * sizeof(double));
-    if (e == cudaSuccess) e = cudaMalloc(&ctx->counts, (kMaxLevels + 1) * sizeof(unsigned long long));
-    // update slots, then one word: the device-side error flag (timed-out waits)
-    if (e == cudaSuccess) e = cudaMalloc(&ctx->upd, (kMaxUpdSlots + 1) * sizeof(unsigned));
-    if (e == cudaSuccess) e = cudaMemset(ctx->upd, 0, (kMaxUpdSlots + 1) * sizeof(unsigned));
+    // the unknown counts; the update slots; one word: the device-side error flag
+    // (timed-out waits)
+    if (e == cudaSuccess) e = cudaMalloc(&ctx->counts, kCountBytes + kUpdBytes);
+    if (e == cudaSuccess) e = cudaMemset(ctx->counts, 0, kCountBytes + kUpdBytes);
+    if (e == cudaSuccess) ctx->upd = reinterpret_cast<unsigned*>(ctx->counts + kMaxLevels + 1);
     if (e == cudaSuccess) e = cudaMalloc(&ctx->cg_sc, 4 * kMaxChannels * sizeof(double));
     if (e == cudaSuccess) e = cudaMalloc(&ctx->dsteps, sizeof(unsigned long long));
     if (e == cudaSuccess) e = cudaMemset(ctx->dsteps, 0, sizeof(unsigned long long));
@@ -1030,7 +1028,6 @@ void di_destroy(di_ctx* ctx) {
     if (ctx->done_ev) cudaEventDestroy(ctx->done_ev);
     if (ctx->norm2) cudaFree(ctx->norm2);
     if (ctx->counts) cudaFree(ctx->counts);
-    if (ctx->upd) cudaFree(ctx->upd);
     if (ctx->cg_sc) cudaFree(ctx->cg_sc);
     if (ctx->dsteps) cudaFree(ctx->dsteps);
     if (ctx->host) cudaFreeHost(ctx->host);

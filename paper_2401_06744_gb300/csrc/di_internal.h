@@ -163,6 +163,10 @@ struct StopState {
     double bnorm2[kMaxChannels];   // ||b||^2 per channel (relative-residual rule)
     double norm2[kMaxChannels];    // ||b - A u||^2 per channel of the last cycle
 };
+// The words that every decode graph clears first: the unknown counts, then the
+// update slots and the timeout flag behind them, one allocation.
+constexpr size_t kCountBytes = (kMaxLevels + 1) * sizeof(unsigned long long);
+constexpr size_t kUpdBytes = (kMaxUpdSlots + 1) * sizeof(unsigned);
 
 // Stop rule parameters (rule: the DI_STOP_* value of the configuration).
 struct StopParams {
@@ -186,12 +190,14 @@ struct PlanParams {
 
 // Levels in use and branch values of the decode from the unknown counts
 // (counts[1 + l]: unknown pixels of level l); initialises *st.
-cudaError_t launch_plan(const unsigned long long* counts, StopState* st, const PlanParams& p,
-                        cudaStream_t s);
+cudaError_t launch_plan(const unsigned long long* counts, StopState* st, StopState* host,
+                        const PlanParams& p, cudaStream_t s);
 // The stop test after one V-cycle: reads and clears the update slots
 // (upd[0 .. nslots-1]; upd[kMaxUpdSlots] is the timeout flag), updates *st
-// and sets the loop handle to 0 once the decode is done.
-cudaError_t launch_stop(unsigned* upd, StopState* st, const StopParams& p,
+// and sets the loop handle to 0 once the decode is done.  host (pinned, of
+// both): gets the state when the decode is planned and when it is done, so no
+// copy follows the graph.
+cudaError_t launch_stop(unsigned* upd, StopState* st, StopState* host, const StopParams& p,
                         unsigned long long h_loop, cudaStream_t s);
 
 // ---------------------------------------------------------------------------

@@ -3064,7 +3064,7 @@ k_combine(const float* __restrict__ parked, int w, int h, int C, int o, int nbx,
 // ---------------------------------------------------------------------------
 
 __global__ void k_plan(const unsigned long long* __restrict__ counts, StopState* __restrict__ st,
-                       PlanParams p) {
+                       StopState* __restrict__ host, PlanParams p) {
     if (threadIdx.x != 0 || blockIdx.x != 0) return;
     const int L = p.L;
     const unsigned long long unk0 = counts[1];
@@ -3084,18 +3084,20 @@ __global__ void k_plan(const unsigned long long* __restrict__ counts, StopState*
     for (int k = 0; k < kMaxChannels; ++k) st->rel[k] = -1.f;
     const bool empty = unk0 == p.n0;
     st->status = empty ? DI_ERR_EMPTY_MASK : DI_OK;
+    if (!empty && Leff == 0) st->converged = 1;  // every pixel known: u = f
+    *host = *st;  // what the host sees unless a stop test follows
     if (empty) {
         cudaGraphSetConditional(p.h_sel, kSelSkip);
         return;
     }
-    if (Leff == 0) st->converged = 1;  // every pixel known: u = f
     cudaGraphSetConditional(p.h_sel, (unsigned)Leff);
     if (Leff > 0) cudaGraphSetConditional(p.h_loop[Leff], p.max_cycles > 0 ? 1u : 0u);
 }
 
 // The stop test of the host loop, on the device: the same float arithmetic
 // in the same order, so the decisions are identical.
-__global__ void k_stop(unsigned* __restrict__ upd, StopState* __restrict__ st, StopParams p,
+__global__ void k_stop(unsigned* __restrict__ upd, StopState* __restrict__ st,
+                       StopState* __restrict__ host, StopParams p,
                        cudaGraphConditionalHandle h_loop) {
     if (threadIdx.x != 0 || blockIdx.x != 0) return;
     const int cycles = st->cycles + 1;
@@ -3151,6 +3153,7 @@ __global__ void k_stop(unsigned* __restrict__ upd, StopState* __restrict__ st, S
         stop = true;
     }
     for (int k = 0; k < p.nslots; ++k) upd[k] = 0u;
+    if (stop) *host = *st;
     cudaGraphSetConditional(h_loop, stop ? 0u : 1u);
 }
 
@@ -4258,16 +4261,16 @@ cudaError_t launch_oras(const float* u_in, int zero_in, const float* rhs, int rh
     }
 }
 
-cudaError_t launch_plan(const unsigned long long* counts, StopState* st, const PlanParams& p,
-                        cudaStream_t s) {
-    k_plan<<<1, 32, 0, s>>>(counts, st, p);
+cudaError_t launch_plan(const unsigned long long* counts, StopState* st, StopState* host,
+                        const PlanParams& p, cudaStream_t s) {
+    k_plan<<<1, 32, 0, s>>>(counts, st, host, p);
     count();
     return cudaGetLastError();
 }
 
-cudaError_t launch_stop(unsigned* upd, StopState* st, const StopParams& p,
+cudaError_t launch_stop(unsigned* upd, StopState* st, StopState* host, const StopParams& p,
                         unsigned long long h_loop, cudaStream_t s) {
-    k_stop<<<1, 32, 0, s>>>(upd, st, p, (cudaGraphConditionalHandle)h_loop);
+    k_stop<<<1, 32, 0, s>>>(upd, st, host, p, (cudaGraphConditionalHandle)h_loop);
     count();
     return cudaGetLastError();
 }
