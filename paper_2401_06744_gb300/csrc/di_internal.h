@@ -236,7 +236,7 @@ struct BatchSeg {
     const uint32_t* mbits; // pack: bits out; block: the level's packed mask
     unsigned* maxupd;      // prolong, block: the image's update slot (nullable)
     unsigned long long* counter;  // pack: the image's unknown count of this level
-    int zero_in, rhs_zero, iters, nbx, nby, wpr, mode, keep;
+    int zero_in, rhs_zero, iters, nbx, nby, wpr, mode, keep;  // zero_in: one value per launch
     float rtol2;
     // block kernel: the start prolonged from the next coarser level inside the
     // kernel (prolong_into_tile) -- pro_mode 0 none, 1 u_in + P pro_e at

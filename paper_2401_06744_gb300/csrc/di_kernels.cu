@@ -1435,9 +1435,9 @@ struct Smem2W {
 // pb, zero for g = 0) and no select on the row group is left in the stencil: 28
 // lane shuffles per warp and CG step, where the lane = column layout took 42
 // and where shuffles and shared-memory accesses share one pipe.  Tile loads and
-// the write of u are 8-byte words.  4K RGB, overlap 2: 13.6 us per CG step and
-// 202 us for ten (lane = column layout: 16.0 and 229), 178 warp instructions per
-// warp and step (221); with the correction's prolongation 240 us (257).
+// the write of u are 8-byte words.  4K RGB, overlap 2: 13.6 us per CG step
+// (lane = column layout: 16.0), 178 warp instructions per warp and step (221); a
+// task without steps 598 (706).
 struct BlockThread {
     int lane, wi, g, l;
     int cl;      // first of the two columns
@@ -1531,18 +1531,14 @@ __device__ __forceinline__ f2 ld_pair(const float* p) {
 // right-hand side tile (RHS0: 0 off the mask); INT: no row of the block on the
 // image's top or bottom row, so every vertical degree is 2.  A thread walks its
 // columns, so a row's centre is the next row's neighbour; the two columns of a
-// row are a packed pair until the masked result goes to its CG pairs.
+// row are a packed pair until the masked result goes to its CG pairs.  (A zero
+// iterate is a tile of zeros: zero_tiles.)
 template <bool F64, bool RHS0, bool INT, bool EVEN>
 __device__ __forceinline__ void block_residual(f2 (&r)[8], const BlockOp& op,
                                                const BlockThread& bt, const float* tc, int ts,
-                                               const float* bc, int bs, int zero_in, int y0,
-                                               int h) {
+                                               const float* bc, int bs, int y0, int h) {
     f2 rv[8];
-    f2 up = 0ull, cen = 0ull;
-    if (!zero_in) {
-        up = ld_pair<EVEN>(tc - ts);
-        cen = ld_pair<EVEN>(tc);
-    }
+    f2 up = ld_pair<EVEN>(tc - ts), cen = ld_pair<EVEN>(tc);
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
         f2 v = 0ull;
@@ -1550,28 +1546,26 @@ __device__ __forceinline__ void block_residual(f2 (&r)[8], const BlockOp& op,
             v = ld_pair<EVEN>(bc);
             bc += bs;
         }
-        if (!zero_in) {
-            const float l = tc[-1], rt = tc[2];
-            tc += ts;
-            const f2 dn = ld_pair<EVEN>(tc);
-            f2 nd = op.nd;
-            if (!INT) {
-                const int gy = y0 + bt.r0 + bt.dr * j;
-                const float e = (float)((gy == 0) + (gy == h - 1));
-                nd = add2(nd, pk(e, e));
-            }
-            if (F64) {
-                const float b0 = lo2(v), b1 = hi2(v);
-                v = pk(res_f64(b0, lo2(nd), lo2(cen), lo2(up), lo2(dn), l, hi2(cen)),
-                       res_f64(b1, hi2(nd), hi2(cen), hi2(up), hi2(dn), lo2(cen), rt));
-            } else {
-                const f2 nb = add2(add2(up, dn), pk(l + hi2(cen), lo2(cen) + rt));
-                const f2 t = fma2(nd, cen, nb);  // -(A u)
-                v = RHS0 ? t : add2(v, t);
-            }
-            up = cen;
-            cen = dn;
+        const float l = tc[-1], rt = tc[2];
+        tc += ts;
+        const f2 dn = ld_pair<EVEN>(tc);
+        f2 nd = op.nd;
+        if (!INT) {
+            const int gy = y0 + bt.r0 + bt.dr * j;
+            const float e = (float)((gy == 0) + (gy == h - 1));
+            nd = add2(nd, pk(e, e));
         }
+        if (F64) {
+            const float b0 = lo2(v), b1 = hi2(v);
+            v = pk(res_f64(b0, lo2(nd), lo2(cen), lo2(up), lo2(dn), l, hi2(cen)),
+                   res_f64(b1, hi2(nd), hi2(cen), hi2(up), hi2(dn), lo2(cen), rt));
+        } else {
+            const f2 nb = add2(add2(up, dn), pk(l + hi2(cen), lo2(cen) + rt));
+            const f2 t = fma2(nd, cen, nb);  // -(A u)
+            v = RHS0 ? t : add2(v, t);
+        }
+        up = cen;
+        cen = dn;
         rv[j] = v;
     }
 #pragma unroll
@@ -1750,17 +1744,25 @@ __device__ __forceinline__ float shared_part(float d, float v, float u, bool fir
     return d == 1.f || first ? __fmaf_rn(d, v, u) : __fmul_rn(d, v);
 }
 
+// The tiles of a launch whose iterate is zero, which no copy fills: zeros, so
+// that the code of every task is the same (the tests per row in the residual and
+// the write were 24 branches and 92 of 690 instructions of a task without CG
+// steps: decode of 4K RGB 1571 -> 1513 us, four in flight 4740 -> 4540).
+__device__ __forceinline__ void zero_tiles(float* s_u, int t, int nt) {
+    for (int i = t; i < 2 * Smem2W::USTRIDE; i += nt) s_u[i] = 0.f;
+}
+
 // The write of 0/1 weights (overlap 2): each pixel is written by the one block
-// whose weight is 1 there, with u_in (the tile; zero_in: 0) added.  up: u_out
+// whose weight is 1 there, with u_in (the tile) added.  up: u_out
 // at local row 0, column cl; us: its step to the next local row; own0, own1:
 // the columns are the block's own; rows: bit j of a local row j of its own
-// (ALL: rows 1 .. 7 are); vec: up is at an 8-byte boundary in every row.  vmax
+// (ALL: rows 1 .. 7 are); VEC: up is at an 8-byte boundary in every row.  vmax
 // gains the largest |x| written.  A lane with one column of its own stores a
 // word, the others two, without a branch on it.
-template <bool ALL>
-__device__ __forceinline__ void block_write01(const f2 (&x)[8], const float* tc, int ts,
-                                              int zero_in, float* up, ptrdiff_t us, bool own0,
-                                              bool own1, uint32_t rows, bool vec, float& vmax) {
+template <bool ALL, bool VEC>
+__device__ __forceinline__ void block_write01_t(const f2 (&x)[8], const float* tc, int ts,
+                                                float* up, ptrdiff_t us, bool own0, bool own1,
+                                                uint32_t rows, float& vmax) {
     const bool two = own0 && own1, one = own0 != own1;
     float m0 = 0.f, m1 = 0.f;
     const int oc = own0 ? 0 : 1;
@@ -1768,10 +1770,9 @@ __device__ __forceinline__ void block_write01(const f2 (&x)[8], const float* tc,
     for (int j = 0; j < 8; ++j) {
         const bool ok = (ALL && j > 0) || ((rows >> j) & 1u);
         const float v0 = block_value(x, 0, j), v1 = block_value(x, 1, j);
-        f2 u = 0ull;
-        if (!zero_in) u = ld_pair<true>(tc);
+        const f2 u = ld_pair<true>(tc);
         const float a = lo2(u) + v0, b = hi2(u) + v1;
-        if (vec) {
+        if (VEC) {
             if (ok && two) *reinterpret_cast<f2*>(up) = pk(a, b);
             if (ok && one) up[oc] = own0 ? a : b;
         } else {
@@ -1787,6 +1788,13 @@ __device__ __forceinline__ void block_write01(const f2 (&x)[8], const float* tc,
     }
     if (own0) vmax = fmaxf(vmax, m0);
     if (own1) vmax = fmaxf(vmax, m1);
+}
+__device__ __forceinline__ void block_write01(const f2 (&x)[8], bool all, const float* tc, int ts,
+                                              float* up, ptrdiff_t us, bool own0, bool own1,
+                                              uint32_t rows, bool vec, float& vmax) {
+    if (all && vec) block_write01_t<true, true>(x, tc, ts, up, us, own0, own1, rows, vmax);
+    else if (vec) block_write01_t<false, true>(x, tc, ts, up, us, own0, own1, rows, vmax);
+    else block_write01_t<false, false>(x, tc, ts, up, us, own0, own1, rows, vmax);
 }
 
 // The start of an iteration formed by prolongation inside a block's tile
@@ -2097,6 +2105,10 @@ k_oras_2w(const float* __restrict__ u_in, int zero_in, const float* __restrict__
     int blk = chan_inner ? (int)blockIdx.x : (int)blockIdx.x / C;
     int ch = chan_inner ? 0 : (int)blockIdx.x - blk * C;
     if (blk >= nblk) return;  // block-uniform
+    if (zero_in) {
+        zero_tiles(s_u, t, 64);
+        __syncthreads();
+    }
     if (use_tma) {
         if (t == 0) {
             for (int b = 0; b < 2; ++b)
@@ -2197,23 +2209,18 @@ k_oras_2w(const float* __restrict__ u_in, int zero_in, const float* __restrict__
         f2 x[8], r[8];
         constexpr bool EV = OV != 2;
         if (y0 > 0 && y0 + B < h) {
-            if (rhs_zero) block_residual<F64, true, true, EV>(r, op, bt, tc, ts, bc, bs, zero_in, y0, h);
-            else block_residual<F64, false, true, EV>(r, op, bt, tc, ts, bc, bs, zero_in, y0, h);
+            if (rhs_zero) block_residual<F64, true, true, EV>(r, op, bt, tc, ts, bc, bs, y0, h);
+            else block_residual<F64, false, true, EV>(r, op, bt, tc, ts, bc, bs, y0, h);
         } else {
-            if (rhs_zero) block_residual<F64, true, false, EV>(r, op, bt, tc, ts, bc, bs, zero_in, y0, h);
-            else block_residual<F64, false, false, EV>(r, op, bt, tc, ts, bc, bs, zero_in, y0, h);
+            if (rhs_zero) block_residual<F64, true, false, EV>(r, op, bt, tc, ts, bc, bs, y0, h);
+            else block_residual<F64, false, false, EV>(r, op, bt, tc, ts, bc, bs, y0, h);
         }
         nsteps += block_cg(x, r, op, bt, iters, rtol2, sh);
 
         float* up = u_out + ch * n + (size_t)(y0 + bt.r0) * w + x0 + bt.cl;
         const ptrdiff_t us = bt.dr * (ptrdiff_t)w;
         if constexpr (OV == 0) {
-            if (op.full)
-                block_write01<true>(x, tc, ts, zero_in, up, us, wx0 > 0.f, wx1 > 0.f, rows_w, vec,
-                                    vmax);
-            else
-                block_write01<false>(x, tc, ts, zero_in, up, us, wx0 > 0.f, wx1 > 0.f, rows_w, vec,
-                                     vmax);
+            block_write01(x, op.full, tc, ts, up, us, wx0 > 0.f, wx1 > 0.f, rows_w, vec, vmax);
         } else {
             // the weighted part of shared pixels is parked in the block's tile
             // for k_combine; the first contributor of a shared pixel (smallest
@@ -2229,7 +2236,7 @@ k_oras_2w(const float* __restrict__ u_in, int zero_in, const float* __restrict__
                 const float wy = s_wy[ly];
                 const float d0 = wx0 * wy, d1 = wx1 * wy;
                 const float v0 = block_value(x, 0, j), v1 = block_value(x, 1, j);
-                const f2 u = zero_in ? 0ull : ld_pair<EV>(tc + j * ts);
+                const f2 u = ld_pair<EV>(tc + j * ts);
                 const bool yf = !(ky > 0 && ly >= first && ly < last);
                 const float a = shared_part(d0, v0, lo2(u), xf0 && yf);
                 const float b = shared_part(d1, v1, hi2(u), xf1 && yf);
@@ -3637,6 +3644,7 @@ k_batch_oras(const BatchSeg* __restrict__ segs, int nseg, int nunits, int split,
                          :: "r"((unsigned)__cvta_generic_to_shared(&s_bar[k])) : "memory");
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
+    if (segs[cur.seg].zero_in) zero_tiles(s_u, t, 64);  // of every segment of the launch
     // no thread may probe a barrier before it is initialised
     __syncthreads();
     prefetch(cur, 0, true);
@@ -3674,7 +3682,7 @@ k_batch_oras(const BatchSeg* __restrict__ segs, int nseg, int nunits, int split,
 
         const BatchSeg& sg = segs[cur.seg];
         const int w = sg.w, h = sg.h, nbx = sg.nbx, nby = sg.nby;
-        const int zero_in = sg.zero_in, rhs_zero = sg.rhs_zero;
+        const int rhs_zero = sg.rhs_zero;
         const size_t n = (size_t)w * h;
         if (cur.seg != cur_seg) {
             // the image changes: flush the previous image's largest update
@@ -3724,14 +3732,14 @@ k_batch_oras(const BatchSeg* __restrict__ segs, int nseg, int nunits, int split,
         f2 x[8], r[8];
         if (y0 > 0 && y0 + B < h) {
             if (rhs_zero)
-                block_residual<false, true, true, true>(r, op, bt, tc, ts, bc, bs_b, zero_in, y0, h);
+                block_residual<false, true, true, true>(r, op, bt, tc, ts, bc, bs_b, y0, h);
             else
-                block_residual<false, false, true, true>(r, op, bt, tc, ts, bc, bs_b, zero_in, y0, h);
+                block_residual<false, false, true, true>(r, op, bt, tc, ts, bc, bs_b, y0, h);
         } else {
             if (rhs_zero)
-                block_residual<false, true, false, true>(r, op, bt, tc, ts, bc, bs_b, zero_in, y0, h);
+                block_residual<false, true, false, true>(r, op, bt, tc, ts, bc, bs_b, y0, h);
             else
-                block_residual<false, false, false, true>(r, op, bt, tc, ts, bc, bs_b, zero_in, y0, h);
+                block_residual<false, false, false, true>(r, op, bt, tc, ts, bc, bs_b, y0, h);
         }
         block_cg(x, r, op, bt, sg.iters, sg.rtol2, sh);
 
@@ -3739,11 +3747,7 @@ k_batch_oras(const BatchSeg* __restrict__ segs, int nseg, int nunits, int split,
         const bool vec = (w & 1) == 0 && (reinterpret_cast<uintptr_t>(uo) & 7) == 0;
         float* up = uo + cur.ch * n + (size_t)(y0 + bt.r0) * w + x0 + bt.cl;
         const ptrdiff_t us = bt.dr * (ptrdiff_t)w;
-        if (op.full)
-            block_write01<true>(x, tc, ts, zero_in, up, us, wx0 > 0.f, wx1 > 0.f, rows_w, vec, vmax);
-        else
-            block_write01<false>(x, tc, ts, zero_in, up, us, wx0 > 0.f, wx1 > 0.f, rows_w, vec,
-                                 vmax);
+        block_write01(x, op.full, tc, ts, up, us, wx0 > 0.f, wx1 > 0.f, rows_w, vec, vmax);
         if (!more) break;
         g = g2;
         cur = nxt;
