@@ -1737,11 +1737,24 @@ __device__ __forceinline__ float block_value(const f2 (&x)[8], int c, int j) {
     return j < 4 ? lo2(x[4 * c + j]) : hi2(x[4 * c + j - 4]);
 }
 
+// Stores under a predicate (written out: left to the compiler they become
+// branches around each store).
+__device__ __forceinline__ void st_if(bool ok, float* p, float a) {
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %2, 0;\n\t"
+                 "@p st.global.f32 [%0], %1;\n\t}" ::"l"(p), "f"(a), "r"((unsigned)ok) : "memory");
+}
+__device__ __forceinline__ void st_pair_if(bool ok, float* p, float a, float b) {
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %3, 0;\n\t"
+                 "@p st.global.v2.f32 [%0], {%1, %2};\n\t}"
+                 ::"l"(p), "f"(a), "f"(b), "r"((unsigned)ok) : "memory");
+}
+
 // What a block of weight d stores of a pixel: u_in + v where the pixel is its
-// own (d = 1), its weighted part elsewhere, the first contributor's with u_in.
-// Every rounding explicit, so that each block kernel gets the same bits.
+// own (d = 1), its weighted part elsewhere, the first contributor's (which a
+// weight of 1 implies) with u_in.  Every rounding explicit, so that each block
+// kernel gets the same bits.
 __device__ __forceinline__ float shared_part(float d, float v, float u, bool first) {
-    return d == 1.f || first ? __fmaf_rn(d, v, u) : __fmul_rn(d, v);
+    return __fmaf_rn(d, v, first ? u : 0.f);
 }
 
 // The tiles of a launch whose iterate is zero, which no copy fills: zeros, so
@@ -2226,32 +2239,42 @@ k_oras_2w(const float* __restrict__ u_in, int zero_in, const float* __restrict__
             // for k_combine; the first contributor of a shared pixel (smallest
             // block index along each shared axis) also carries u_in, so the
             // combine pass only adds
-            const int first = shared_first(o), last = first + shared_per_seam(o);
-            const bool xf0 = !(kx > 0 && bt.cl >= first && bt.cl < last);
-            const bool xf1 = !(kx > 0 && bt.cl + 1 >= first && bt.cl + 1 < last);
-            float* const mine = parked + ((size_t)blk * C + ch) * (B * B) + bt.cl;
+            // A column's class and, in a row of weight 1, where it goes are the
+            // thread's; everything per row is a select or a predicate (branches
+            // around the stores took 10 % of a launch without CG steps)
+            const int first = shared_first(o), nsh = shared_per_seam(o);
+            const bool xf0 = !(kx > 0 && bt.cl >= first && bt.cl < first + nsh);
+            const bool xf1 = !(kx > 0 && bt.cl + 1 >= first && bt.cl + 1 < first + nsh);
+            const bool z0 = wx0 > 0.f, z1 = wx1 > 0.f, own0 = wx0 == 1.f, own1 = wx1 == 1.f;
+            const bool both = z0 && z1, same = both && own0 == own1 && (vec || !own0);
+            float* part = parked + ((size_t)blk * C + ch) * (B * B) + bt.r0 * B + bt.cl;
+            const float* tu = tc;
+            float m0 = 0.f, m1 = 0.f;
 #pragma unroll
             for (int j = 0; j < 8; ++j) {
                 const int ly = bt.r0 + bt.dr * j;
                 const float wy = s_wy[ly];
-                const float d0 = wx0 * wy, d1 = wx1 * wy;
+                const bool rz = wy > 0.f, rp = wy == 1.f;
+                const bool yf = !(ky > 0 && (unsigned)(ly - first) < (unsigned)nsh);
                 const float v0 = block_value(x, 0, j), v1 = block_value(x, 1, j);
-                const f2 u = ld_pair<EV>(tc + j * ts);
-                const bool yf = !(ky > 0 && ly >= first && ly < last);
-                const float a = shared_part(d0, v0, lo2(u), xf0 && yf);
-                const float b = shared_part(d1, v1, hi2(u), xf1 && yf);
-                float* const dst = up + j * us;
-                float* const part = mine + ly * B;
-                float* const pa = d0 == 1.f ? dst : part;
-                if (d0 > 0.f && d1 > 0.f && (d0 == 1.f) == (d1 == 1.f) && (vec || d0 < 1.f)) {
-                    *reinterpret_cast<float2*>(pa) = make_float2(a, b);
-                } else {
-                    if (d0 > 0.f) pa[0] = a;
-                    if (d1 > 0.f) (d1 == 1.f ? dst : part)[1] = b;
-                }
-                if (d0 > 0.f) vmax = fmaxf(vmax, fabsf(v0));
-                if (d1 > 0.f) vmax = fmaxf(vmax, fabsf(v1));
+                const f2 u = ld_pair<EV>(tu);
+                // weight 1 implies the first contributor
+                const float a = shared_part(wx0 * wy, v0, lo2(u), xf0 && yf);
+                const float b = shared_part(wx1 * wy, v1, hi2(u), xf1 && yf);
+                float* const pa = rp && own0 ? up : part;
+                float* const pb = rp && own1 ? up : part;
+                const bool two = rp ? same : rz && both;
+                st_pair_if(two, pa, a, b);
+                st_if(rz && z0 && !two, pa, a);
+                st_if(rz && z1 && !two, pb + 1, b);
+                m0 = fmaxf(m0, rz ? fabsf(v0) : 0.f);
+                m1 = fmaxf(m1, rz ? fabsf(v1) : 0.f);
+                up += us;
+                part += bt.dr * B;
+                tu += ts;
             }
+            if (z0) vmax = fmaxf(vmax, m0);
+            if (z1) vmax = fmaxf(vmax, m1);
         }
         if (!more) break;
         blk = nb2;
