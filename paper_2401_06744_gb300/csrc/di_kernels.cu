@@ -1398,7 +1398,7 @@ struct Tile2W {
 
 // Shared-memory layout of the FP32 kernel (floats, from a 128-byte aligned
 // base): two u tiles of TH rows with pitch PU (a 40-wide TMA box, or the
-// 34-wide cp.async copy at column 0), the row weights, with a prolongation
+// 34-wide cp.async copy at column 1), the row weights, with a prolongation
 // two patches of 18 x 18 coarse cells, then two right-hand side tiles of B
 // rows with pitch PB (36-wide TMA box).  Tile strides are multiples of 128
 // bytes, the alignment of a TMA destination.
@@ -4338,7 +4338,7 @@ cudaError_t launch_restrict(const float* u, const float* b, int rhs_zero, const 
     // GPU's threads (at 960x540 cells both forms take 10.3 us, at 1920x1080 28.9
     // against 36.8)
     if (su == kF32 && sb == kF32 && sr == kF32 && !f64 && C > 1 &&
-        (long long)wH * hH >= 152LL * 2048) {
+        (long long)wH * hH >= 152LL * 2048 && hH <= 4 * 65535) {  // grid rows of 4
         const dim3 b1(32, 4), g1 = grid2(wH, hH, b1);
         auto* const kern = C == 2   ? (vec ? k_restrict_c<2, true> : k_restrict_c<2, false>)
                            : C == 3 ? (vec ? k_restrict_c<3, true> : k_restrict_c<3, false>)
