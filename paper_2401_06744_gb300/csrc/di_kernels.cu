@@ -21,7 +21,7 @@
 //                    TMA; optionally the start formed by prolongation inside it
 //   k_oras_4w        the same with four warps per (block, channel), for launches of
 //                    few local problems (the same bits)
-//   k_oras_2w_h, k_oras_4w_h  the same two with FP16 / BF16 local iterates
+//   k_oras_2w_h      k_oras_2w with FP16 / BF16 local iterates
 //   k_oras_warp      8x8 and 16x16 blocks: one warp per (block, channel)
 //   k_combine        Algorithm 2 step 3 for pixels shared by several blocks: the
 //                    sums of their weighted contributions in a fixed order
@@ -3025,258 +3025,6 @@ k_oras_2w_h(const TU* __restrict__ u_in, int zero_in, const TU* __restrict__ rhs
     }
 }
 
-// ---- four warps per block, 16-bit iterates --------------------------------------
-// k_oras_2w_h for launches of few local problems, with the threads of oras_4w: a
-// column of eight rows per thread.  The rows that other warps hold are advanced
-// by the same 16-bit operations as in their own warps.
-// Decode of 1280x720 RGB with FP16 local solves: 711 -> 647 us.
-template <class H, class TU>
-__global__ void __launch_bounds__(128, 4)
-k_oras_4w_h(const TU* __restrict__ u_in, int zero_in, const TU* __restrict__ rhs, int rhs_zero,
-            const uint32_t* __restrict__ mbits, int wpr, int w, int h, int C, int o, int nbx,
-            int nby, float alpha, int iters, float rtol2, TU* __restrict__ u_out,
-            float* __restrict__ parked, unsigned* __restrict__ maxupd,
-            const __grid_constant__ CUtensorMap tm_u, const __grid_constant__ CUtensorMap tm_b,
-            int use_tma, unsigned* __restrict__ errflag,
-            unsigned long long* __restrict__ step_count) {
-    typedef typename H::T2 T2;
-    constexpr bool kF = std::is_same<TU, float>::value;
-    constexpr int B = 32, TH = Smem2W::TH, P = Smem2W::PU, PB = Smem2W::PB;
-    __shared__ __align__(128) float s_u[Smem2W::USTRIDE];
-    __shared__ __align__(128) float s_b[Smem2W::BSTRIDE];
-    __shared__ float s_wy[B], s_row0[2][32], s_row7[4][32], s_mx[4];
-    __shared__ float4 s_red1, s_red2;
-    __shared__ __align__(8) unsigned long long s_bar;
-
-    const int t = threadIdx.x, lane = t & 31, wrp = t >> 5;
-    const int wi = wrp >> 1, g = wrp & 1;
-    const int r0 = wi ? (g ? 16 : 31) : (g ? 15 : 0), dr = wi == g ? 1 : -1;
-    const int s = B - o;
-    const int blk = (int)blockIdx.x / C, ch = (int)blockIdx.x - blk * C;
-    const int ky = blk / nbx, kx = blk - ky * nbx, x0 = kx * s, y0 = ky * s;
-    const size_t n = (size_t)w * h;
-    const unsigned bar = (unsigned)__cvta_generic_to_shared(&s_bar);
-
-    if (kF && use_tma) {
-        if (t == 0) {
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar) : "memory");
-            asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-            const unsigned bytes = (zero_in ? 0u : (unsigned)Smem2W::TMA_U_BYTES) +
-                                   (rhs_zero ? 0u : (unsigned)Smem2W::TMA_B_BYTES);
-            asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;"
-                         :: "r"(bar), "r"(bytes) : "memory");
-            if (!zero_in)
-                tma_load_3d((unsigned)__cvta_generic_to_shared(s_u), &tm_u, (x0 - 1) & ~3, y0 - 1,
-                            ch, bar);
-            if (!rhs_zero)
-                tma_load_3d((unsigned)__cvta_generic_to_shared(s_b), &tm_b, x0 & ~3, y0, ch, bar);
-        }
-    } else {
-        // every load of a thread before its first store
-        const TU* su = u_in + ch * n;
-        const TU* sb = rhs + ch * n;
-        const int gxa = x0 - 1 + lane, gxb = gxa + 32;
-        float ra[9], rb[9], vb[8];
-#pragma unroll
-        for (int i = 0; i < 9; ++i) {
-            const int ty = wrp + 4 * i, gy = y0 - 1 + ty;
-            const bool rok = !zero_in && ty < TH && gy >= 0 && gy < h;
-            ra[i] = rok && gxa >= 0 && gxa < w ? ldf(su + (ptrdiff_t)gy * w + gxa) : 0.f;
-            rb[i] = rok && lane < TH - 32 && gxb < w ? ldf(su + (ptrdiff_t)gy * w + gxb) : 0.f;
-        }
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {
-            const int gy = y0 + wrp + 4 * i;
-            vb[i] = !rhs_zero && x0 + lane < w && gy < h ? ldf(sb + (size_t)gy * w + x0 + lane)
-                                                         : 0.f;
-        }
-#pragma unroll
-        for (int i = 0; i < 9; ++i) {
-            const int ty = wrp + 4 * i;
-            if (ty < TH) {
-                s_u[ty * P + 1 + lane] = ra[i];
-                if (lane < TH - 32) s_u[ty * P + 33 + lane] = rb[i];
-            }
-        }
-#pragma unroll
-        for (int i = 0; i < 8; ++i) s_b[(wrp + 4 * i) * PB + lane] = vb[i];
-    }
-
-    // the local operator of the thread's column
-    uint32_t rowm = 0xffffffffu;
-    {
-        const int gy = y0 + r0 + dr * lane;
-        if (lane < 8 && gy < h) {
-            const uint32_t* row = mbits + (size_t)gy * wpr + (x0 >> 5);
-            rowm = __funnelshift_r(__ldg(row), __ldg(row + 1), x0 & 31);
-        }
-    }
-    const int bw = min(B, w - x0), bh = min(B, h - y0);
-    const int gx = x0 + lane;
-    const float hc = (lane > 0 ? 1.f : (gx > 0 ? alpha : 0.f)) +
-                     (lane + 1 < bw ? 1.f : (gx < w - 1 ? alpha : 0.f));
-    T2 nd[4], keep[4];
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        float d[2], kp[2];
-#pragma unroll
-        for (int e = 0; e < 2; ++e) {
-            const int j = k + 4 * e, ly = r0 + dr * j, gy = y0 + ly;
-            const float vc = (ly > 0 ? 1.f : (gy > 0 ? alpha : 0.f)) +
-                             (ly + 1 < bh ? 1.f : (gy < h - 1 ? alpha : 0.f));
-            d[e] = -(hc + vc);
-            kp[e] = ((__shfl_sync(kFull, rowm, j) >> lane) & 1u) ? 0.f : 1.f;
-        }
-        nd[k] = H::make(d[0], d[1]);
-        keep[k] = H::make(kp[0], kp[1]);
-    }
-    const int odd = lane & 1, outer = odd ? lane + 1 : lane - 1;
-    const float mo = (lane == 0 || lane == 31) ? 0.f : 1.f;
-    const T2 mo2 = H::make(mo, mo);
-    const float inv_o1 = o > 1 ? 1.f / (float)(o - 1) : 0.f;
-    const float wx = gx < w ? ramp_weight(lane, kx, nbx, s, o, inv_o1) : 0.f;
-    if (t < B) s_wy[t] = lane < bh ? ramp_weight(lane, ky, nby, s, o, inv_o1) : 0.f;
-
-    __syncthreads();  // the mbarrier is initialised, or the tiles are there
-    const bool tma = kF && use_tma;
-    if (tma) {
-        const bool ok = mbar_wait(bar, 0u);
-        if (__syncthreads_or(!ok)) {
-            if (!ok) mbar_wait(bar, 0u);  // one more bounded wait before the CTA leaves
-            if (t == 0 && errflag) atomicExch(errflag, 1u);
-            return;
-        }
-    }
-    const int du = tma ? ((x0 - 1) & 3) : 1, db = tma ? (x0 & 3) : 0;
-    const float* const tc = s_u + du + (r0 + 1) * P + lane + 1;  // local row 0
-    const int ts = dr * P;
-
-    // FP32 residual, then its maximum for the normalisation
-    float rv[8];
-    float mx = 0.f;
-    {
-        const float* bc = s_b + db + r0 * PB + lane;
-        const float dh = (float)((gx > 0) + (gx < w - 1)) + 2.f;
-#pragma unroll
-        for (int j = 0; j < 8; ++j) {
-            float v = rhs_zero ? 0.f : bc[j * dr * PB];
-            if (!zero_in) {
-                const float* c0 = tc + j * ts;
-                const int gy = y0 + r0 + dr * j;
-                const float e = (float)((gy == 0) + (gy == h - 1));
-                v = res_stencil<false>(v, dh - e, c0[0], c0[-ts], c0[ts], c0[-1], c0[1]);
-            }
-            v *= j < 4 ? H::lo(keep[j]) : H::hi(keep[j - 4]);
-            rv[j] = v;
-            mx = fmaxf(mx, fabsf(v));
-        }
-    }
-    mx = warp_max(mx);
-    if (lane == 0) s_mx[wrp] = mx;
-    __syncthreads();
-    mx = fmaxf(fmaxf(s_mx[0], s_mx[1]), fmaxf(s_mx[2], s_mx[3]));
-    const float sc = mx > 0.f ? mx / H::kScale : 1.f;  // r = sc * r_narrow
-    const float isc = 1.f / sc;
-
-    auto block_sum4 = [&](f2 acc, float4* red) {
-        float v = lo2(acc) + hi2(acc);
-        v = warp_sum(v);
-        if (lane == 0) reinterpret_cast<float*>(red)[wrp] = v;
-        __syncthreads();
-        const float4 a = *red;
-        return (a.x + a.y) + (a.z + a.w);
-    };
-    T2 x[4], r[4], p[4], q[4];
-    auto publish = [&]() {
-        if (g) s_row0[wi][lane] = H::lo(r[0]);
-        s_row7[wrp][lane] = H::hi(r[3]);
-    };
-    f2 acc = 0ull;
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        r[k] = H::make(rv[k] * isc, rv[k + 4] * isc);
-        p[k] = r[k];
-        x[k] = H::make(0.f, 0.f);
-        const f2 rw = H::wide(r[k]);
-        acc = fma2(rw, rw, acc);
-    }
-    publish();
-    float rr = block_sum4(acc, &s_red2);
-    // local rows -1 and 8 of p
-    T2 edge = H::make(g ? s_row0[wi ^ 1][lane] : 0.f, s_row7[wrp ^ 1][lane]);
-    const float rr_stop = fmaxf(rtol2 >= 0.f ? fmaxf(rtol2, 1e-14f) * rr
-                                             : fmaxf(1e-14f * rr, -rtol2 * isc * isc),
-                                FLT_MIN);
-    bool bad = !(rr < INFINITY);
-    unsigned nsteps = 0;
-    for (int it = 0; it < iters; ++it) {
-        if (!(rr > rr_stop) || bad) break;  // identical in the four warps
-        acc = 0ull;
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            const T2 in = __shfl_xor_sync(kFull, p[k], 1);
-            const T2 ou = __shfl_sync(kFull, p[k], outer);
-            const T2 up = k > 0 ? p[k - 1] : H::make(H::lo(edge), H::lo(p[3]));
-            const T2 dn = k < 3 ? p[k + 1] : H::make(H::hi(p[0]), H::hi(edge));
-            T2 nb = __hadd2(up, dn);
-            nb = __hadd2(nb, in);
-            nb = __hfma2(mo2, ou, nb);
-            q[k] = __hmul2(__hfma2(nd[k], p[k], nb), keep[k]);  // -(A_i p), 0 on the mask
-            acc = fma2(H::wide(p[k]), H::wide(q[k]), acc);
-        }
-        const float pq = -block_sum4(acc, &s_red1);
-        if (!(pq >= FLT_MIN) || !(pq < INFINITY)) {
-            bad = !(pq < INFINITY) || pq != pq;
-            break;
-        }
-        const float a = quotient(rr, pq);
-        const T2 a2 = H::make(a, a);
-        acc = 0ull;
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            x[k] = __hfma2(a2, p[k], x[k]);
-            r[k] = __hfma2(a2, q[k], r[k]);
-            const f2 rw = H::wide(r[k]);
-            acc = fma2(rw, rw, acc);
-        }
-        publish();
-        const float rrn = block_sum4(acc, &s_red2);
-        if (!(rrn < INFINITY)) { bad = true; break; }
-        const float beta = quotient(rrn, rr);
-        rr = rrn;
-        const T2 b2 = H::make(beta, beta);
-#pragma unroll
-        for (int k = 0; k < 4; ++k) p[k] = __hfma2(b2, p[k], r[k]);
-        edge = __hfma2(b2, edge, H::make(g ? s_row0[wi ^ 1][lane] : 0.f, s_row7[wrp ^ 1][lane]));
-        ++nsteps;
-    }
-
-    float vmax = 0.f;
-    const float vs = bad ? 0.f : sc;  // a non-finite narrow iterate gives no correction
-    const int first = shared_first(o), last = first + shared_per_seam(o);
-    const bool xf = !(kx > 0 && lane >= first && lane < last);
-    TU* const up = u_out + ch * n + (size_t)(y0 + r0) * w + gx;
-    float* const mine = parked + ((size_t)blk * C + ch) * (B * B) + lane;
-    const ptrdiff_t us = dr * (ptrdiff_t)w;
-#pragma unroll
-    for (int j = 0; j < 8; ++j) {
-        const int ly = r0 + dr * j;
-        const float d = wx * s_wy[ly];
-        const float v = (j < 4 ? H::lo(x[j]) : H::hi(x[j - 4])) * vs;
-        const float u = zero_in ? 0.f : tc[j * ts];
-        const bool yf = !(ky > 0 && ly >= first && ly < last);
-        const float a = shared_part(d, v, u, xf && yf);
-        if (d == 1.f) stf(up + j * us, a);
-        else if (d > 0.f) mine[ly * B] = a;
-        if (d > 0.f) vmax = fmaxf(vmax, fabsf(v));
-    }
-    if (step_count && t == 0) atomicAdd(step_count, (unsigned long long)nsteps);
-    if (maxupd) {
-        vmax = warp_max(vmax);
-        if (lane == 0 && vmax > 0.f) atomicMax(maxupd, __float_as_uint(vmax));
-    }
-}
-
 // The sums of the pixels that several blocks share (overlap 1 or >= 3), in the
 // fixed order upper left, upper right, lower left, lower right; the first term
 // carries u_in.  A warp takes one part of a (block, channel): blockIdx.z = 0 the
@@ -4095,25 +3843,6 @@ cudaError_t launch_oras_2w(const float* u_in, int zero_in, const float* rhs, int
                                   alpha, iters, rtol2, u_out, parked, maxupd, chan_inner, tm_u,
                                   tm_b, use_tma, errflag, step_count, pro_e, wH, hH, pro_max,
                                   tm_e, use_tma_e);
-    } else if (!f64 && ntasks <= kQuadTasks) {
-        use_tma = stor == kF32 && (!zero_in || !rhs_zero) &&
-                  (zero_in || make_map(&tm_u, u_in, w, h, C, Smem2W::PU, Smem2W::TH)) &&
-                  (rhs_zero || make_map(&tm_b, rhs, w, h, C, Smem2W::PB, B));
-        auto go = [&](auto kern4, auto stored) {
-            typedef decltype(stored) TU;
-            kern4<<<ntasks, 128, 0, s>>>(reinterpret_cast<const TU*>(u_in), zero_in,
-                                         reinterpret_cast<const TU*>(rhs), rhs_zero, mbits, wpr, w,
-                                         h, C, o, nbx, nby, alpha, iters, rtol2,
-                                         reinterpret_cast<TU*>(u_out), parked, maxupd, tm_u, tm_b,
-                                         use_tma, errflag, step_count);
-        };
-        if (precision == 1) {
-            if (stor != kF32) go(k_oras_4w_h<HalfT, __half>, __half());
-            else go(k_oras_4w_h<HalfT, float>, 0.f);
-        } else {
-            if (stor != kF32) go(k_oras_4w_h<Bf16T, __nv_bfloat16>, __nv_bfloat16());
-            else go(k_oras_4w_h<Bf16T, float>, 0.f);
-        }
     } else {
 #define DI_ORAS_H(H, TU, F)                                                                     \
     run_oras_2w_h<H, TU, F>(grid, smem, s, u_in, zero_in, rhs, rhs_zero, mbits, wpr, w, h, C, o, \

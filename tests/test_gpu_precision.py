@@ -144,33 +144,3 @@ def test_fp64_restriction_matches_oracle_more_closely(di):
     assert out[1] <= out[0] + 1e-7
     # FP64 arithmetic, one rounding to FP32 at the end: within one FP32 ulp
     assert out[1] <= float(np.abs(ref).max()) * 2.0 ** -23
-
-
-@pytest.mark.parametrize("prec,eps", [("fp16", 2.0 ** -11), ("bf16", 2.0 ** -8)])
-@pytest.mark.parametrize("h,w,o,aligned", [(31, 40, 2, True), (70, 96, 6, True), (129, 63, 6, True),
-                                           (97, 130, 2, False), (64, 64, 3, True),
-                                           (190, 124, 2, True)])
-def test_narrow_iteration_of_few_problems(di, prec, eps, h, w, o, aligned):
-    # launches of few local problems (four warps each): within the rounding of
-    # the 16-bit steps of the oracle's K-step CG.  Bound: K steps of at most
-    # about ten operations, each rounded to eps of the block's largest correction.
-    K = 6
-    code = {"fp16": di.PREC_FP16, "bf16": di.PREC_BF16}[prec]
-    g = np.random.default_rng(h + w + o)
-    c = (g.random((h, w)) < 0.1).astype(np.uint8)
-    c[0, 0] = 1
-    f = g.uniform(0, 255, (1, h, w)).astype(np.float32)
-    u = np.where(c.astype(bool), f, g.uniform(0, 255, f.shape)).astype(np.float32)
-    ref = M.oras_iteration(u, M.rhs(f, c), c, 32, o, 0.5, ("cg", K))
-    scale = np.abs(ref - u).max()
-    flat = torch.empty(u.size + 1, dtype=torch.float32, device=DEV)
-    ut = (flat[:-1] if aligned else flat[1:]).view(u.shape)
-    ut.copy_(torch.from_numpy(u))
-    with di.Context(precision=code, overlap=o) as ctx:
-        out = ctx.oras_iteration(ut, torch.from_numpy(f).to(DEV), torch.from_numpy(c).to(DEV), K,
-                                 rhs_zero=True)
-        torch.cuda.synchronize()
-    out = out.cpu().numpy()
-    assert np.isfinite(out).all()
-    assert np.array_equal(out[:, c == 1], u[:, c == 1])
-    assert np.abs(out - ref).max() <= 10 * K * eps * scale + 2e-4
