@@ -105,8 +105,10 @@ inline size_t oras_scratch_floats(int w, int h, int C, int B, int o) {
 // mbits: the packed mask of this level).  Each local CG runs `iters` steps or
 // until r.r <= max(rtol2, 1e-14) * (r.r)_0 (rtol2 >= 0), or until
 // r.r <= max(1e-14 (r.r)_0, -rtol2) (rtol2 < 0: an absolute level, per block
-// and channel, summed over the block's pixels).  max |v_i| over pixels with
-// nonzero weight is folded into *maxupd (nullable).
+// and channel, summed over the block's pixels); 32x32 blocks with FP32
+// iterates solve residuals whose r.r or p.Ap would underflow scaled by a power
+// of two (kTinyNorm2).  max |v_i| over pixels with nonzero weight is folded
+// into *maxupd (nullable).
 // ev (nullable): two events recorded on `s` right before and right after the
 // block kernel (the combine kernels follow the second one).  precision: 0
 // FP32, 1 FP16, 2 BF16 local CG iterates (32x32 blocks; other sizes use FP32).

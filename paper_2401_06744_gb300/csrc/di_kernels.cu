@@ -1583,11 +1583,27 @@ struct BlockShared {
 };
 
 // a / b for normal b > 0: one approximate reciprocal (both warps of a block
-// compute it from the same words, so they agree).
+// compute it from the same words, so they agree).  0 for b > 2^126, as with a
+// fast division.
 __device__ __forceinline__ float quotient(float a, float b) {
     float r;
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(b));
     return a * r;
+}
+
+// Residuals whose squared norm lies below kTinyNorm2 are solved scaled by
+// kTinyScale, their solution scaled back: both powers of two, so the local
+// solve of a scaled image has the bits of the image's own.  Without it r.r and
+// p.Ap of values of 1e-17 and less would underflow before the relative stop
+// (1e-14 of the first r.r) is reached.  Squares of kTinyScale times such a
+// residual stay below 2^96.  The test costs the 4K RGB iteration 1 us of 187.
+constexpr float kTinyNorm2 = 0x1p-64f, kTinyScale = 0x1p80f;
+__device__ __forceinline__ bool tiny_residual(float rr, float rtol2) {
+    return rr < kTinyNorm2 && !(rtol2 < 0.f && rr <= -rtol2);  // that stops at once
+}
+// -rtol2 (an absolute level of r.r) of a residual scaled by kTinyScale.
+__device__ __forceinline__ float tiny_rtol2(float rtol2) {
+    return rtol2 < 0.f ? (rtol2 * kTinyScale) * kTinyScale : rtol2;
 }
 
 // Sum over a warp of the two-warp form, the row groups last, so that the
@@ -1601,7 +1617,8 @@ __device__ __forceinline__ float warp_sum_block(float v) {
 // Up to `iters` CG steps on A_i x = r from x = 0 (r is overwritten); both
 // warps of the block.  rtol2 >= 0: relative stop (r.r <= max(rtol2, 1e-14)
 // (r.r)_0); rtol2 < 0: also stop once r.r <= -rtol2 (an absolute level, or the
-// FP32 floor).  The last step updates x alone.  Returns the completed steps.
+// FP32 floor).  Tiny residuals are scaled (kTinyScale).  The last step updates
+// x alone.  Returns the completed steps.
 // Bound by the register file: an instruction takes half a cycle per 32-bit
 // operand word it reads (a packed FMA of three distinct pairs 3 cycles, an
 // add 2, a scalar add 1), which is why nothing here trades fewer
@@ -1629,6 +1646,28 @@ __device__ __forceinline__ unsigned block_cg_t(f2 (&x)[8], f2 (&r)[8], const Blo
     float rr = sh.red2[0] + sh.red2[1];
     float2 pb = make_float2(0.f, 0.f);  // local row -1 of p
     if (bt.g) pb = sh.seam[bt.wi ^ 1][bt.l];
+    const bool tiny = tiny_residual(rr, rtol2);
+    if (tiny) {  // the same in both warps
+        const f2 up = pk(kTinyScale, kTinyScale);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            r[i] = mul2(r[i], up);
+            p[i] = r[i];
+            if (i == 0) acc0 = mul2(r[i], r[i]);
+            else if (i == 4) acc1 = mul2(r[i], r[i]);
+            else if (i < 4) acc0 = fma2(r[i], r[i], acc0);
+            else acc1 = fma2(r[i], r[i], acc1);
+        }
+        acc0 = add2(acc0, acc1);
+        part = warp_sum_block(lo2(acc0) + hi2(acc0));
+        if (bt.lane == 0) sh.red1[bt.wi] = part;
+        __syncthreads();
+        rr = sh.red1[0] + sh.red1[1];
+        __syncthreads();  // the first step writes red1
+        pb.x *= kTinyScale;
+        pb.y *= kTinyScale;
+        rtol2 = tiny_rtol2(rtol2);
+    }
     // never below the smallest normal, so that the quotients stay finite
     const float rr_stop = fmaxf(rtol2 >= 0.f ? fmaxf(rtol2, 1e-14f) * rr : fmaxf(1e-14f * rr, -rtol2),
                                 FLT_MIN);
@@ -1712,6 +1751,11 @@ __device__ __forceinline__ unsigned block_cg_t(f2 (&x)[8], f2 (&r)[8], const Blo
             pb.x = fmaf(beta, pb.x, sv.x);
             pb.y = fmaf(beta, pb.y, sv.y);
         }
+    }
+    if (tiny) {
+        const f2 down = pk(1.f / kTinyScale, 1.f / kTinyScale);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) x[i] = mul2(x[i], down);
     }
     return (unsigned)it;
 }
@@ -2552,6 +2596,21 @@ __device__ __forceinline__ void oras_4w(
     float rr = block_sum4(acc, &s_red2);
     float pb = g ? s_row0[wi ^ 1][lane] : 0.f;  // local row -1 of p
     float p8 = s_row7[wrp ^ 1][lane];           // local row 8
+    const bool tiny = tiny_residual(rr, rtol2);
+    if (tiny) {  // the same in every warp
+        const f2 up = pk(kTinyScale, kTinyScale);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            r[k] = mul2(r[k], up);
+            p[k] = r[k];
+            acc = k ? fma2(r[k], r[k], acc) : mul2(r[k], r[k]);
+        }
+        rr = block_sum4(acc, &s_red1);
+        __syncthreads();  // the first step writes s_red1
+        pb *= kTinyScale;
+        p8 *= kTinyScale;
+        rtol2 = tiny_rtol2(rtol2);
+    }
     const float rr_stop = fmaxf(rtol2 >= 0.f ? fmaxf(rtol2, 1e-14f) * rr : fmaxf(1e-14f * rr, -rtol2),
                                 FLT_MIN);
     int it = 0;
@@ -2593,6 +2652,11 @@ __device__ __forceinline__ void oras_4w(
         for (int k = 0; k < 4; ++k) p[k] = fma2(b2, p[k], r[k]);
         if (g) pb = fmaf(beta, pb, s_row0[wi ^ 1][lane]);
         p8 = fmaf(beta, p8, s_row7[wrp ^ 1][lane]);
+    }
+    if (tiny) {
+        const f2 down = pk(1.f / kTinyScale, 1.f / kTinyScale);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) x[k] = mul2(x[k], down);
     }
 
     // the weighted write (k_oras_2w)

@@ -328,6 +328,28 @@ def test_oras_few_problems_same_bits(di, h, w, o, aligned, rhs_zero):
             assert np.array_equal(a[0], b4[ch])
 
 
+@pytest.mark.parametrize("C,o", [(1, 2), (1, 6), (4, 2), (4, 6), (4, 5)])
+@pytest.mark.parametrize("rhs_zero", [True, False])
+def test_oras_of_a_scaled_image(di, C, o, rhs_zero):
+    # the iteration is linear and powers of two are exact, so an image scaled by
+    # one has the bits of the image's own result, also where the squares of its
+    # residual are no normal FP32 numbers (2^-76 and below) or are none at all;
+    # one channel takes four warps per local problem, four channels two
+    h, w = 500, 600
+    f, _, c = _case(h, w, C, 0.06, 77 + o, nan=False)
+    g = np.random.default_rng(o)
+    known = c.astype(bool)
+    u = np.where(known, f, g.uniform(0, 255, f.shape)).astype(np.float32)
+    b = g.normal(size=f.shape).astype(np.float32)
+    with di.Context(block=32, overlap=o, alpha=0.5) as ctx:
+        ref = N(ctx.oras_iteration(T(u), T(b), T(c), 12, rhs_zero=rhs_zero))
+        assert np.abs(ref - u).max() > 1
+        for e in (20, 40, -20, -40, -60, -76, -90, -100):
+            k = np.float32(2.0 ** e)
+            out = N(ctx.oras_iteration(T(u * k), T(b * k), T(c), 12, rhs_zero=rhs_zero))
+            assert np.array_equal(out, ref * k), e
+
+
 @pytest.mark.parametrize("w", [16, 48, 64, 112, 4112])
 @pytest.mark.parametrize("h", [1, 31, 33, 130])
 def test_packed_mask_sixteen_columns_at_a_time(di, h, w):
