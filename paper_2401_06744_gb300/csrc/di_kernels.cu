@@ -4410,12 +4410,12 @@ cudaError_t launch_batch_oras(const BatchSeg* segs, int nseg, int nunits, int nt
                               int o, float alpha,
                               const BatchState& bs, cudaStream_t s) {
     if (nunits < 1 || nseg < 1) return cudaSuccess;
+    if (shared_per_seam(o) != 0) return cudaErrorInvalidValue;  // 0/1 weights only
     if (ntasks <= kQuadTasks) {  // as for one image
         k_batch_oras_4w<<<nunits * cmax, 128, 0, s>>>(segs, nseg, cmax, o, alpha, bs);
         count();
         return cudaGetLastError();
     }
-    if (shared_per_seam(o) != 0) return cudaErrorInvalidValue;  // 0/1 weights only
     int nsm = 0;
     const size_t smem = Smem2W::bytes(true, true);
     const int oc = cached_occupancy((const void*)k_batch_oras, 64, smem, smem, &nsm);

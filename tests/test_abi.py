@@ -93,3 +93,20 @@ def test_plan_counts_narrow_coarse_storage(di):
     coarse = sum(w * h for (w, h) in p32["sizes"][1:]) * 3
     slack = 3 * 256 * p32["levels"]  # per-buffer alignment
     assert abs(p32["workspace_bytes"] - p16["workspace_bytes"] - 3 * 2 * coarse) <= slack
+
+
+@pytest.mark.parametrize("ntasks", [1, 608, 609, 5000])
+@pytest.mark.parametrize("o", [1, 3, 16])
+def test_batched_block_kernel_refuses_shared_pixels(di, o, ntasks):
+    # its write takes every weight for 0 or 1: overlaps with other weights are
+    # refused before either form of the kernel is launched (without a device only:
+    # there a launch that gets through fails, and no kernel sees these arguments)
+    torch = pytest.importorskip("torch")
+    if torch.cuda.is_available():
+        pytest.skip("needs a machine without a GPU")
+    fn = getattr(ctypes.CDLL(di.LIB_PATH),
+                 "_ZN2di17launch_batch_orasEPKNS_8BatchSegEiiiiifRKNS_10BatchStateEP11CUstream_st")
+    fn.argtypes = [ctypes.c_void_p] + 5 * [ctypes.c_int] + [ctypes.c_float] + 2 * [ctypes.c_void_p]
+    state = ctypes.create_string_buffer(1024)  # a zero BatchState, not read
+    invalid_value = 1  # cudaErrorInvalidValue; a launch without a device gives another error
+    assert fn(None, 1, ntasks, ntasks, 1, o, 0.5, ctypes.addressof(state), None) == invalid_value
