@@ -24,7 +24,8 @@
 //   k_oras_2w_h      k_oras_2w with FP16 / BF16 local iterates
 //   k_oras_warp      8x8 and 16x16 blocks: one warp per (block, channel)
 //   k_combine        Algorithm 2 step 3 for pixels shared by several blocks: the
-//                    sums of their weighted contributions in a fixed order
+//                    sums of their weighted contributions in a fixed order;
+//                    k_combine_px for blocks of 8 and 16
 //   k_plan, k_stop   the device-driven decode: levels in use and start, and the
 //                    stop test after every V-cycle (conditional graph nodes)
 //   k_batch_*        the batched form: the same steps over the segment tables of
@@ -3091,9 +3092,9 @@ k_oras_2w_h(const TU* __restrict__ u_in, int zero_in, const TU* __restrict__ rhs
 
 // The sums of the pixels that several blocks share (overlap 1 or >= 3), in the
 // fixed order upper left, upper right, lower left, lower right; the first term
-// carries u_in.  A warp takes one part of a (block, channel): blockIdx.z = 0 the
-// seam left of the block (two blocks), 1 the seam above it (two), 2 the corner
-// where they cross (four).  One launch per iteration instead of a row and a
+// carries u_in; for 32x32 blocks.  A warp takes one part of a (block, channel):
+// blockIdx.z = 0 the seam left of the block (two blocks), 1 the seam above it
+// (two), 2 the corner where they cross (four).  One launch per iteration instead of a row and a
 // column pass: with the parts in tiles by block, a warp reaches all its
 // addresses from one block index.  Bound by latency (one dependent load round
 // trip per warp, four rows in flight), not bytes: that is why the parts go to
@@ -3101,10 +3102,11 @@ k_oras_2w_h(const TU* __restrict__ u_in, int zero_in, const TU* __restrict__ rhs
 // on 1920x1080 RGB went from 116 to 107 us, a decode of that size from 1.38 to
 // 1.20 ms and one of 481x321 RGB from 1.05 to 0.91 ms (one warp for all three
 // parts: 1.22 ms and no gain at 481x321).
-template <class TU, int B>
+template <class TU>
 __global__ void __launch_bounds__(256)
 k_combine(const float* __restrict__ parked, int w, int h, int C, int o, int nbx, int nby,
           TU* __restrict__ u_out) {
+    constexpr int B = 32;
     const int lane = threadIdx.x & 31;
     const int unit = (int)blockIdx.x * 8 + (int)(threadIdx.x >> 5);  // kx * C + ch
     if (unit >= nbx * C) return;
@@ -3139,9 +3141,9 @@ k_combine(const float* __restrict__ parked, int w, int h, int C, int o, int nbx,
             add2_rows(lf, (ky > 0 ? wlo : 0) + i0, ky < nby - 1 ? whi : min(B, h - y0) - 1, di,
                       first + j);
     } else if (blockIdx.z == 1) {
-        const int x = lane & (B - 1);
+        const int x = lane;
         if (ky > 0 && x >= (kx > 0 ? wlo : 0) && x <= (kx < nbx - 1 ? whi : min(B, w - x0) - 1))
-            add2_rows(up, first + lane / B, first + nsh - 1, 32 / B, x);
+            add2_rows(up, first, first + nsh - 1, 1, x);
     } else if (kx > 0 && ky > 0 && j < nsh) {
         const float* ul = up - (size_t)C * (B * B) + s;
         const int x = first + j;
@@ -3149,6 +3151,61 @@ k_combine(const float* __restrict__ parked, int w, int h, int C, int o, int nbx,
             stf(dst + (size_t)i * w + x,
                 ul[i * B + x] + up[i * B + x] + lf[i * B + x] + me[i * B + x]);
     }
+}
+
+// The same sums for blocks of 8 and 16, where a part of a block is a run of a few
+// pixels and most lanes of its warp would idle: a thread per column and
+// kCombineRows rows of pixels.  Bound by the sectors of the tiles (a word of
+// each).  ORAS iteration of 8 steps, 3840x2160 RGB, against k_combine's warps:
+// 8x8 blocks at overlap 4 2958 -> 2207 us, at overlap 1 988 -> 774; 16x16 at
+// overlap 4 637 -> 604, at overlap 8 1337 -> 1174 (eight rows per thread: 1185).
+// With 32x32 blocks, whose parts fill their warps, k_combine is the better one
+// (overlap 4: 272 against 306).
+constexpr int kCombineRows = 4;
+template <int B>
+__global__ void __launch_bounds__(256)
+k_combine_px(const float* __restrict__ parked, int w, int h, int C, int o, int nbx, int nby,
+             float* __restrict__ u_out) {
+    const int x = blockIdx.x * 32 + threadIdx.x, ch = blockIdx.z;
+    const int y0 = (blockIdx.y * 8 + threadIdx.y) * kCombineRows;
+    if (x >= w || y0 >= h) return;
+    const int s = B - o, first = shared_first(o), last = first + shared_per_seam(o);
+    // the block whose own stride holds the coordinate (the lower one of a
+    // shared pixel); local coordinate 0 has weight 0 there (overlap >= 3)
+    int kx = min(x / s, nbx - 1), lx = x - kx * s;
+    const bool sx = kx > 0 && lx >= first && lx < last;
+    if (!sx && kx > 0 && lx == 0) {
+        --kx;
+        lx = s;
+    }
+    int ky = min(y0 / s, nby - 1), ly = y0 - ky * s;
+    const size_t row = (size_t)nbx * C * (B * B);  // tiles of a row of blocks
+    const int lf = s - C * (B * B);                // the same pixel in the left block's tile
+    const ptrdiff_t up = s * B - (ptrdiff_t)row;   // and in the upper block's
+    const float* col = parked + ((size_t)kx * C + ch) * (B * B) + lx;
+    float v[kCombineRows];
+    unsigned put = 0;
+#pragma unroll
+    for (int r = 0; r < kCombineRows; ++r) {
+        const bool sy = ky > 0 && ly >= first && ly < last;
+        const bool top = !sy && ky > 0 && ly == 0;  // weight 0: the upper block's row s
+        const float* me = col + (size_t)(top ? ky - 1 : ky) * row + (top ? s : ly) * B;
+        v[r] = 0.f;
+        if (y0 + r < h && (sx || sy)) {
+            put |= 1u << r;
+            v[r] = sx && sy ? me[up + lf] + me[up] + me[lf] + me[0]
+                   : sx     ? me[lf] + me[0]
+                            : me[up] + me[0];
+        }
+        if (++ly == s && ky < nby - 1) {
+            ++ky;
+            ly = 0;
+        }
+    }
+    float* dst = u_out + ((size_t)ch * h + y0) * w + x;
+#pragma unroll
+    for (int r = 0; r < kCombineRows; ++r)
+        if ((put >> r) & 1u) dst[(size_t)r * w] = v[r];
 }
 
 // ---------------------------------------------------------------------------
@@ -3967,14 +4024,19 @@ cudaError_t launch_combine(const float* parked, int w, int h, int C, int o, int 
     // Overlap 2 gives 0/1 weights: no pixel is shared, nothing to add.
     if (shared_per_seam(o) == 0 || nbx * nby == 1) return cudaSuccess;
     const dim3 grid((unsigned)((nbx * C + 7) / 8), (unsigned)nby, 3);
-    if (stor == kF16)
-        k_combine<__half, B><<<grid, 256, 0, s>>>(parked, w, h, C, o, nbx, nby,
-                                                  reinterpret_cast<__half*>(u_out));
+    constexpr int kRows = 8 * kCombineRows;  // of a CTA of k_combine_px
+    if constexpr (B < 32)  // FP32 only
+        k_combine_px<B><<<dim3((unsigned)((w + 31) / 32), (unsigned)((h + kRows - 1) / kRows),
+                               (unsigned)C),
+                          dim3(32, 8), 0, s>>>(parked, w, h, C, o, nbx, nby, u_out);
+    else if (stor == kF16)
+        k_combine<__half><<<grid, 256, 0, s>>>(parked, w, h, C, o, nbx, nby,
+                                               reinterpret_cast<__half*>(u_out));
     else if (stor == kBF16)
-        k_combine<__nv_bfloat16, B><<<grid, 256, 0, s>>>(parked, w, h, C, o, nbx, nby,
-                                                         reinterpret_cast<__nv_bfloat16*>(u_out));
+        k_combine<__nv_bfloat16><<<grid, 256, 0, s>>>(parked, w, h, C, o, nbx, nby,
+                                                      reinterpret_cast<__nv_bfloat16*>(u_out));
     else
-        k_combine<float, B><<<grid, 256, 0, s>>>(parked, w, h, C, o, nbx, nby, u_out);
+        k_combine<float><<<grid, 256, 0, s>>>(parked, w, h, C, o, nbx, nby, u_out);
     count();
     return cudaGetLastError();
 }

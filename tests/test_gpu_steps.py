@@ -288,6 +288,21 @@ def test_oras_block_edges(di, h, w, o):
                               out)
 
 
+@pytest.mark.parametrize("h,w", [(9, 17), (31, 33), (32, 95), (36, 64), (63, 40), (101, 130)])
+@pytest.mark.parametrize("B,o", [(8, 1), (8, 3), (8, 4), (16, 1), (16, 3), (16, 5), (16, 8)])
+def test_oras_shared_pixels_of_small_blocks(di, h, w, B, o):
+    # the sums of pixels shared by blocks of 8 and 16, at ragged last blocks and
+    # at the edges of a thread's four rows and a warp's 32 columns: against the
+    # oracle's K-step CG (the bound of test_oras_iteration_matches_oracle_cg)
+    f, fn, c = _case(h, w, 2, 0.07, 3 * h + w + B + o)
+    g = np.random.default_rng(h * w)
+    u = np.where(c.astype(bool), f, g.uniform(0, 255, f.shape)).astype(np.float32)
+    with di.Context(block=B, overlap=o, alpha=0.4) as ctx:
+        out = N(ctx.oras_iteration(T(u), T(fn), T(c), 4, rhs_zero=True))
+    ref = M.oras_iteration(u, M.rhs(f, c), c, B, o, 0.4, ("cg", 4))
+    assert np.abs(out - ref).max() < 1e-3 * np.abs(ref - u).max() + 2e-4
+
+
 QUAD_CASES = [  # (h, w, overlap, aligned): up to 608 local problems in one channel, more in four
     (601, 600, 2, True), (500, 601, 6, True), (601, 640, 4, False), (660, 580, 2, False),
 ]
