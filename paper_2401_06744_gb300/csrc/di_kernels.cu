@@ -601,7 +601,9 @@ k_reduce_slot(const double* __restrict__ partials, int nparts, double* __restric
 // as TU, the right-hand side b as TB, rH as TO (FP16/BF16 on the coarse levels
 // in the 16-bit precision modes).  F64: the children's residuals are formed
 // and summed in FP64 (the finest-grid refinement residual) and rounded once.
-template <bool VEC, class TU, class TB, class TO, bool F64>
+// BESIDE (for VEC): the patch is loaded beside the cell's mask byte, not after
+// it, and dropped if the cell is known.
+template <bool VEC, class TU, class TB, class TO, bool F64, bool BESIDE = false>
 __device__ __forceinline__ void restrict_body(const TU* __restrict__ u, const TB* __restrict__ b, int rhs_zero,
            int w, int h, const uint8_t* __restrict__ cH, TO* __restrict__ rH, int wH,
            int hH, int bx, int by, int bz) {
@@ -617,10 +619,11 @@ __device__ __forceinline__ void restrict_body(const TU* __restrict__ u, const TB
     if (VEC && X >= 1 && Y >= 1 && 2 * X + 2 < w && 2 * Y + 2 < h) {
         // a cell whose 4x4 patch lies inside the image (all but the border
         // cells): every child has four neighbours and the count is 4, so the
-        // same sums as below without a bounds test (the same bits).  The
-        // patch is loaded beside the cell's mask byte, not after it: the
-        // kernel waits for memory, and known cells, whose sum is dropped, are
-        // few and their rows are the neighbours' rows too
+        // same sums as below without a bounds test (the same bits)
+        if (!BESIDE && known) {
+            stf(rH + ch * nH + P, 0.f);
+            return;
+        }
         const TU* r0 = uc + (size_t)y0 * w + x0;
         float t[4][4];
 #pragma unroll
@@ -699,28 +702,48 @@ __device__ __forceinline__ void restrict_body(const TU* __restrict__ u, const TB
     stf(rH + ch * nH + P, (float)(sum * (R)(4 >> (cnt >> 1))));
 }
 
-// The large levels of FP32 images of several channels: one thread per coarse
-// cell and all its channels, every channel's patch in flight together.  The
-// kernel waits for memory, so what counts is loads in flight: CTAs of 128
-// threads, eight per SM at 64 registers (a few spilled: still better than three
-// CTAs of 256 at 77 registers, 34.5 us).  3840x2160 RGB (127 MB, 19 us at the
-// copy rate): 41.1 us with a thread per cell and channel and the patch loaded
-// after the mask byte, 36.8 loaded beside it, 28.9 here; with a right-hand side
-// 49 and 39.7.  VEC: children pairs as 8-byte words.  Border cells as above.
-template <int C, bool VEC>
-__global__ void __launch_bounds__(128, 8)
-k_restrict_c(const float* __restrict__ u, const float* __restrict__ b, int rhs_zero, int w, int h,
+// The large levels of FP32 images: one thread per coarse cell and all its
+// channels, every channel's patch in flight together.  The kernel waits for
+// memory, so what counts is loads in flight: CTAs of 128 threads (gray: 256, the
+// small CTAs come and go too fast where there is nothing to do, 9.4 us against
+// 5.9 at density 0.9), as many per SM as the registers of a thread's patches
+// allow (three channels without a right-hand side 9: 27.7 us, 10: 26.8, 11:
+// 28.4; with one 7: 39.3, 8: 38.2; eight everywhere, with spills: 30.4 and 39.1).
+// The patch is loaded after the cell's mask byte, and not at all for a known
+// cell; the mask bytes are fetched into L2 a wave of CTAs ahead, which gains 1.4
+// us.  (Loaded beside the byte it is as fast where few cells are known, but where
+// nearly all are it took 25.8 and 36.0 us for the 10.3 and 10.5 below.)
+// 3840x2160 RGB (127 MB, 19 us at the copy rate), mask density 0.04 / 0.5 / 0.9:
+// 42.0 / 40.1 / 14.4 us with a thread per cell and channel, 26.8 / 24.6 / 10.3
+// here; with a right-hand side 48.8 / 43.4 / 14.4 and 38.2 / 33.0 / 10.5; gray
+// 15.8 / 14.4 / 6.0 and 12.1 / 11.0 / 5.9.
+// VEC: children pairs as 8-byte words.  Border cells as above.
+__host__ __device__ constexpr int restrict_rows(int C) { return C == 1 ? 8 : 4; }  // of cells per CTA
+constexpr int restrict_ctas(int C, bool vec, bool rhs0) {  // per SM
+    if (C == 1) return 8;
+    return rhs0 ? (C == 2 ? 14 : C == 3 ? (vec ? 10 : 9) : 7) : C == 2 ? 10 : C == 3 ? 8 : 6;
+}
+constexpr int kRestrictAhead = 152 * 8 * 128;  // cells: a wave of CTAs
+template <int C, bool VEC, bool RHS0>
+__global__ void __launch_bounds__(32 * restrict_rows(C), restrict_ctas(C, VEC, RHS0))
+k_restrict_c(const float* __restrict__ u, const float* __restrict__ b, int w, int h,
              const uint8_t* __restrict__ cH, float* __restrict__ rH, int wH, int hH) {
-    const int X = blockIdx.x * 32 + threadIdx.x, Y = blockIdx.y * 4 + threadIdx.y;
+    constexpr int ROWS = restrict_rows(C);
+    const int X = blockIdx.x * 32 + threadIdx.x, Y = blockIdx.y * ROWS + threadIdx.y;
     if (X >= wH || Y >= hH) return;
     const size_t n = (size_t)w * h, nH = (size_t)wH * hH, P = (size_t)Y * wH + X;
+    if (threadIdx.x == 0 && P + kRestrictAhead < nH)
+        asm volatile("prefetch.global.L2 [%0];" ::"l"(cH + P + kRestrictAhead));
     if (X < 1 || Y < 1 || 2 * X + 2 >= w || 2 * Y + 2 >= h) {
         for (int ch = 0; ch < C; ++ch)
-            restrict_body<VEC, float, float, float, false>(u, b, rhs_zero, w, h, cH, rH, wH, hH,
+            restrict_body<VEC, float, float, float, false>(u, b, RHS0, w, h, cH, rH, wH, hH,
                                                            blockIdx.x, blockIdx.y, ch);
         return;
     }
-    const uint8_t known = cH[P];
+    if (cH[P]) {
+        for (int ch = 0; ch < C; ++ch) rH[ch * nH + P] = 0.f;
+        return;
+    }
     auto pair = [](const float* p) {
         return VEC ? *reinterpret_cast<const float2*>(p) : make_float2(p[0], p[1]);
     };
@@ -737,7 +760,7 @@ k_restrict_c(const float* __restrict__ u, const float* __restrict__ b, int rhs_z
             l[ch][j] = p[(size_t)(j + 1) * w - 1];
             r[ch][j] = p[(size_t)(j + 1) * w + 2];
             rb[ch][j] = make_float2(0.f, 0.f);
-            if (!rhs_zero) rb[ch][j] = pair(b + ch * n + at + (size_t)(j + 1) * w);
+            if (!RHS0) rb[ch][j] = pair(b + ch * n + at + (size_t)(j + 1) * w);
         }
     }
 #pragma unroll
@@ -749,20 +772,20 @@ k_restrict_c(const float* __restrict__ u, const float* __restrict__ b, int rhs_z
             const float2 up = mid[ch][j], ce = mid[ch][j + 1], dn = mid[ch][j + 2];
             const float l0 = 4.f * ce.x - (l[ch][j] + ce.y + up.x + dn.x);
             const float l1 = 4.f * ce.y - (ce.x + r[ch][j] + up.y + dn.y);
-            sum += (rhs_zero ? 0.f : rb[ch][j].x) - l0;
-            sum += (rhs_zero ? 0.f : rb[ch][j].y) - l1;
+            sum += (RHS0 ? 0.f : rb[ch][j].x) - l0;
+            sum += (RHS0 ? 0.f : rb[ch][j].y) - l1;
         }
-        rH[ch * nH + P] = known ? 0.f : sum;
+        rH[ch * nH + P] = sum;
     }
 }
 
-template <bool VEC, class TU, class TB, class TO, bool F64>
+template <bool VEC, class TU, class TB, class TO, bool F64, bool BESIDE = false>
 __global__ void __launch_bounds__(256)
 k_restrict(const TU* __restrict__ u, const TB* __restrict__ b, int rhs_zero,
            int w, int h, const uint8_t* __restrict__ cH, TO* __restrict__ rH, int wH,
            int hH) {
-    restrict_body<VEC, TU, TB, TO, F64>(u, b, rhs_zero, w, h, cH, rH, wH, hH, blockIdx.x, blockIdx.y,
-                                        blockIdx.z);
+    restrict_body<VEC, TU, TB, TO, F64, BESIDE>(u, b, rhs_zero, w, h, cH, rH, wH, hH, blockIdx.x,
+                                                blockIdx.y, blockIdx.z);
 }
 
 // Cell-centred bilinear prolongation.  A fine pixel takes 9/16 of its parent
@@ -3382,8 +3405,8 @@ k_batch_grid(const BatchSeg* __restrict__ segs, int nseg, BatchState bs) {
         float* rH = static_cast<float*>(sg.out0);
         if ((w & 1) == 0 && ((reinterpret_cast<uintptr_t>(u) |
                               (sg.rhs_zero ? 0 : reinterpret_cast<uintptr_t>(b))) & 7) == 0)
-            restrict_body<true, float, float, float, false>(u, b, sg.rhs_zero, w, h, cH, rH, wH,
-                                                            hH, bx, by, bz);
+            restrict_body<true, float, float, float, false, true>(u, b, sg.rhs_zero, w, h, cH, rH,
+                                                                  wH, hH, bx, by, bz);
         else
             restrict_body<false, float, float, float, false>(u, b, sg.rhs_zero, w, h, cH, rH, wH,
                                                              hH, bx, by, bz);
@@ -4190,18 +4213,33 @@ cudaError_t launch_restrict(const float* u, const float* b, int rhs_zero, const 
                      ((reinterpret_cast<uintptr_t>(u) |
                        reinterpret_cast<uintptr_t>(rhs_zero ? nullptr : b)) % 8 == 0);
     // one thread for all channels of a cell where the level's cells still fill the
-    // GPU's threads (at 960x540 cells both forms take 10.3 us, at 1920x1080 28.9
-    // against 36.8)
-    if (su == kF32 && sb == kF32 && sr == kF32 && !f64 && C > 1 &&
+    // GPU's threads (three channels, mask density 0.04 / 0.9: at 960x540 cells 7.7 /
+    // 4.0 us against 10.4 / 5.0, at 1920x1080 26.8 / 10.3 against 42.0 / 14.4; at
+    // 480x270 3.9 / 2.3 against 4.1 / 2.5, but with a right-hand side at 0.5 4.4
+    // against 3.8)
+    if (su == kF32 && sb == kF32 && sr == kF32 && !f64 &&
         (long long)wH * hH >= 152LL * 2048 && hH <= 4 * 65535) {  // grid rows of 4
-        const dim3 b1(32, 4), g1 = grid2(wH, hH, b1);
-        auto* const kern = C == 2   ? (vec ? k_restrict_c<2, true> : k_restrict_c<2, false>)
-                           : C == 3 ? (vec ? k_restrict_c<3, true> : k_restrict_c<3, false>)
-                                    : (vec ? k_restrict_c<4, true> : k_restrict_c<4, false>);
-        kern<<<g1, b1, 0, s>>>(u, b, rhs_zero, w, h, cH, rH, wH, hH);
+        const dim3 b1(32, restrict_rows(C)), g1 = grid2(wH, hH, b1);
+#define DI_RESTRICT_C(NC)                                                         \
+    (vec ? (rhs_zero ? k_restrict_c<NC, true, true> : k_restrict_c<NC, true, false>) \
+         : (rhs_zero ? k_restrict_c<NC, false, true> : k_restrict_c<NC, false, false>))
+        auto* const kern = C == 1   ? DI_RESTRICT_C(1)
+                           : C == 2 ? DI_RESTRICT_C(2)
+                           : C == 3 ? DI_RESTRICT_C(3)
+                                    : DI_RESTRICT_C(4);
+#undef DI_RESTRICT_C
+        kern<<<g1, b1, 0, s>>>(u, b, w, h, cH, rH, wH, hH);
     } else if (su == kF32 && sb == kF32 && sr == kF32) {
         if (vec && f64)
             k_restrict<true, float, float, float, true><<<grid, blk, 0, s>>>(
+                u, b, rhs_zero, w, h, cH, rH, wH, hH);
+        else if (vec && (long long)grid.x * grid.y * grid.z <= 152 * 3)
+            // few CTAs: a launch lasts as long as its loads one after the other
+            // (480x270 RGB, mask density 0.04 / 0.9: 2.6 / 2.0 us, after the mask
+            // byte 2.9 / 1.9); larger launches read no patch of a known cell
+            // (960x540 gray 2.6 / 2.0 us, beside the byte 2.4 / 2.3; RGB 4.1 / 2.5,
+            // 3.8 / 3.1)
+            k_restrict<true, float, float, float, false, true><<<grid, blk, 0, s>>>(
                 u, b, rhs_zero, w, h, cH, rH, wH, hH);
         else if (vec)
             k_restrict<true, float, float, float, false><<<grid, blk, 0, s>>>(

@@ -417,6 +417,22 @@ def test_restrict_all_channels_of_a_cell(di, h, w, C, aligned, rhs_zero):
         assert np.array_equal(r[ch], one[0])
 
 
+@pytest.mark.parametrize("h,w,C", [(70, 95, 1), (1101, 1203, 3), (1200, 1100, 4)])
+@pytest.mark.parametrize("density", [0.7, 1.0])
+def test_restrict_of_mostly_known_images(di, h, w, C, density):
+    # known cells give 0, the few others what test_restrict_residual says
+    f, fn, c = _case(h, w, C, density, h + w)
+    cH = M.mask_downsample(c)
+    g = np.random.default_rng(6)
+    u = np.where(c.astype(bool), f, g.uniform(0, 255, f.shape)).astype(np.float32)
+    b = np.where(c.astype(bool), 0.0, g.normal(size=f.shape)).astype(np.float32)
+    for rhs, rhs_zero in ((fn, True), (b, False)):
+        rH = N(di.restrict_residual(T(u), T(rhs), T(c), T(cH), rhs_zero=rhs_zero))
+        ref = M.restrict_residual(M.residual(u, M.rhs(f, c) if rhs_zero else b, c), cH)
+        assert np.abs(rH - ref).max() < 1e-3
+        assert not rH[:, cH == 1].any()
+
+
 PRO_CASES = [  # (h, w, overlap, rhs_zero, aligned)
     (70, 96, 2, True, True), (70, 96, 2, False, False), (70, 96, 6, False, True),
     (33, 35, 2, False, True), (130, 100, 2, True, False), (61, 250, 6, True, True),
