@@ -202,35 +202,36 @@ __global__ void k_values_down(const uint8_t* __restrict__ c, const float* __rest
 // thread forms the mask of its R cells (rows 8 apart): cH = max over the
 // children (four mask bytes, as byte pairs where the image allows), the packed
 // words (known or beyond the image = 1; the last column's CTAs write the
-// padding word too), the count of unknown cells, the child flags in a shared
-// tile with a one-cell halo, and bH = 0 where nothing is known.  Then the
-// known cells, collected in a list, get their mask values (modified or naive
-// downsampling, the weights and sums of values_down_body), a thread each: the
-// flags of the cell and of its four neighbours come from the tile, the known
-// children's values of every channel are loaded together.  values = 0: masks
-// only (a given start).
-// The list is there because the weights are most of the instructions and few
-// cells are known (15 % at a mask density of 4 %): with a thread per cell the
-// kernel was bound by instruction issue (474 warp instructions per 32 cells).
-// 3840x2160 RGB at 4 % (about 10 us at the copy rate): 47.3 -> 22.1 us, at 10 %
-// 51.3 -> 32.8; 1920x1080 RGB 13.3 -> 8.4; 3001x1999 RGB 30.6 -> 16.5.
-template <int R>
+// padding word too), the count of unknown cells, and bH = 0 where nothing is
+// known.  Then the known cells get their mask values (MOD: modified, else naive
+// downsampling, the weights and sums of values_down_body), the known children's
+// values of every channel loaded together.  The modified weights take the child
+// flags of the cell's four neighbours from a shared tile with a one-cell halo.
+// LIST (MOD only): the known cells are collected in a list and get their values
+// a thread each; otherwise each thread does its own.  values = 0: masks only (a
+// given start).
+// The list is there because the modified weights are most of the instructions
+// and few cells are known (15 % at a mask density of 4 %): with a thread per cell
+// the kernel was bound by instruction issue (474 warp instructions per 32 cells).
+// Times of the kernel alone, mask density 0.04 / 0.5 (3840x2160 RGB takes about
+// 10 us at the copy rate), a thread per cell and channel by channel before:
+// 3840x2160 RGB 49.5 / 51.4 -> 26.6 / 36.1 us, 1920x1080 RGB 12.3 / 13.0 -> 7.9 /
+// 11.5, 3001x1999 RGB 35.6 / 37.5 -> 20.4 / 28.5.
+template <int R, bool LIST, bool MOD>
 __device__ __forceinline__ void pyramid_level_body(
     const uint8_t* __restrict__ c, const float* __restrict__ b, int w, int h, int C,
-    uint8_t* __restrict__ cH, float* __restrict__ bH, int wH, int hH, int modified, int values,
+    uint8_t* __restrict__ cH, float* __restrict__ bH, int wH, int hH, int values,
     uint32_t* __restrict__ bits, int wpr, unsigned long long* __restrict__ unknown, int bx,
     int by, int nbx) {
+    static_assert(MOD || !LIST, "the naive average needs no list");
     constexpr int ROWS = 8 * R;
     const int tx = threadIdx.x, ty = threadIdx.y, t = ty * 32 + tx;
     const int X0 = bx * 32, Y0 = by * ROWS, X = X0 + tx;
     const size_t nH = (size_t)wH * hH;
-    __shared__ uint8_t s_kn[ROWS + 2][34];   // child flags (bit k: child k known)
-    __shared__ uint16_t s_list[32 * ROWS];   // known cells, 32 row + column
-    __shared__ unsigned s_n, s_u;
-    if (t == 0) {
-        s_n = 0u;
-        s_u = 0u;
-    }
+    __shared__ uint8_t s_kn[MOD ? ROWS + 2 : 1][34];   // child flags (bit k: child k known)
+    __shared__ uint16_t s_list[LIST ? 32 * ROWS : 1];  // known cells, 32 row + column
+    __shared__ unsigned s_n, s_unk[8];
+    if (LIST && t == 0) s_n = 0u;
     // flags of the children of coarse cell (Xc, Yc), 0 off the level
     const bool pairs = (w & 1) == 0 && (reinterpret_cast<uintptr_t>(c) & 1) == 0;
     auto children = [&](int Xc, int Yc) -> unsigned {
@@ -258,59 +259,28 @@ __device__ __forceinline__ void pyramid_level_body(
     unsigned ck[R];
 #pragma unroll
     for (int r = 0; r < R; ++r) ck[r] = children(X, Y0 + ty + 8 * r);
-    if (values && modified) {  // the halo (uniform over the grid)
+    if (MOD && values) {  // the halo (uniform over the grid)
         if (ty == 0) s_kn[0][tx + 1] = (uint8_t)children(X, Y0 - 1);
         if (ty == 7) s_kn[ROWS + 1][tx + 1] = (uint8_t)children(X, Y0 + ROWS);
         for (int i = t; i < 2 * ROWS; i += 256)
             s_kn[(i >> 1) + 1][(i & 1) ? 33 : 0] =
                 (uint8_t)children((i & 1) ? X0 + 32 : X0 - 1, Y0 + (i >> 1));
     }
-    __syncthreads();
-    unsigned unk = 0;
-#pragma unroll
-    for (int r = 0; r < R; ++r) {
-        const int ly = ty + 8 * r, Y = Y0 + ly;
-        const bool kn = ck[r] != 0u, in = X < wH && Y < hH;
-        const unsigned word = __ballot_sync(kFull, X >= wH || kn);
-        if (Y < hH && tx == 0) {
-            bits[(size_t)Y * wpr + bx] = word;
-            if (bx == nbx - 1) bits[(size_t)Y * wpr + wpr - 1] = 0xffffffffu;  // the padding word
-        }
-        if (Y < hH) unk += (unsigned)__popc(~word);  // warp-uniform
-        if (in) cH[(size_t)Y * wH + X] = kn ? 1 : 0;
-        if (values) {
-            s_kn[ly + 1][tx + 1] = (uint8_t)ck[r];
-            const unsigned list = __ballot_sync(kFull, kn);
-            unsigned at = 0;
-            if (tx == 0 && list) at = atomicAdd(&s_n, (unsigned)__popc(list));
-            at = __shfl_sync(kFull, at, 0);
-            if (kn) {
-                s_list[at + (unsigned)__popc(list & ((1u << tx) - 1u))] = (uint16_t)(32 * ly + tx);
-            } else if (in) {
-                for (int ch = 0; ch < C; ++ch) bH[ch * nH + (size_t)Y * wH + X] = 0.f;
-            }
-        }
-    }
-    if (unknown && tx == 0 && unk) atomicAdd(&s_u, unk);
-    __syncthreads();
-    if (unknown && t == 0 && s_u) atomicAdd(unknown, (unsigned long long)s_u);
-    if (!values) return;
+    if constexpr (LIST) __syncthreads();  // s_n
     const size_t n = (size_t)w * h;
-    const unsigned known = s_n;
-    for (unsigned i = t; i < known; i += 256) {
-        const int e = s_list[i], lx = e & 31, ly = e >> 5;
-        const unsigned f = s_kn[ly + 1][lx + 1];
+    auto value = [&](auto channels, int lx, int ly, unsigned f) {  // of a known cell with the flags f
+        constexpr int NC = decltype(channels)::value;  // C <= NC
         const int Xc = X0 + lx, Yc = Y0 + ly;
         const float* bp = b + (size_t)(2 * Yc) * w + 2 * Xc;
-        float bv[kMaxChannels][4];
+        float bv[NC][4];
 #pragma unroll
-        for (int ch = 0; ch < kMaxChannels; ++ch)
+        for (int ch = 0; ch < NC; ++ch)
 #pragma unroll
             for (int k = 0; k < 4; ++k)
-                bv[ch][k] = ch < C && ((f >> k) & 1u)
+                bv[ch][k] = (NC == 1 || ch < C) && ((f >> k) & 1u)
                                 ? bp[ch * n + (k >> 1) * (size_t)w + (k & 1)] : 0.f;
         unsigned side[2] = {0u, 0u}, vert[2] = {0u, 0u};  // neighbours known: left, right; above, below
-        if (modified) {
+        if (MOD) {
             // the flags are 0 off the level; the child columns and rows off an
             // odd image have no neighbour across the cell either, but they are
             // unknown and get no weight
@@ -325,7 +295,7 @@ __device__ __forceinline__ void pyramid_level_body(
         for (int k = 0; k < 4; ++k) {
             const unsigned m = ((f >> (k ^ 1)) & 1u) + ((f >> (k ^ 2)) & 1u) + side[k & 1] +
                                vert[k >> 1];
-            wt[k] = !((f >> k) & 1u) ? 0.f : modified ? (float)(4 - (int)m) : 1.f;
+            wt[k] = !((f >> k) & 1u) ? 0.f : MOD ? (float)(4 - (int)m) : 1.f;
             den += wt[k];
         }
         if (den == 0.f) {  // gap of the printed rule: the naive average
@@ -336,23 +306,76 @@ __device__ __forceinline__ void pyramid_level_body(
         const float inv = 1.f / fmaxf(1.f, den);
         const size_t P = (size_t)Yc * wH + Xc;
 #pragma unroll
-        for (int ch = 0; ch < kMaxChannels; ++ch) {
+        for (int ch = 0; ch < NC; ++ch) {
             float num = 0.f;
 #pragma unroll
             for (int k = 0; k < 4; ++k)
                 if (wt[k] != 0.f) num = __fmaf_rn(wt[k], bv[ch][k], num);
-            if (ch < C) bH[ch * nH + P] = num * inv;
+            if (NC == 1 || ch < C) bH[ch * nH + P] = num * inv;
         }
+    };
+    unsigned unk = 0;
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        const int ly = ty + 8 * r, Y = Y0 + ly;
+        const bool kn = ck[r] != 0u, in = X < wH && Y < hH;
+        const unsigned word = __ballot_sync(kFull, X >= wH || kn);
+        if (Y < hH && tx == 0) {
+            bits[(size_t)Y * wpr + bx] = word;
+            if (bx == nbx - 1) bits[(size_t)Y * wpr + wpr - 1] = 0xffffffffu;  // the padding word
+        }
+        if (Y < hH) unk += (unsigned)__popc(~word);  // warp-uniform
+        if (in) cH[(size_t)Y * wH + X] = kn ? 1 : 0;
+        if (values) {
+            if (MOD) s_kn[ly + 1][tx + 1] = (uint8_t)ck[r];
+            if constexpr (LIST) {
+                const unsigned list = __ballot_sync(kFull, kn);
+                unsigned at = 0;
+                if (tx == 0 && list) at = atomicAdd(&s_n, (unsigned)__popc(list));
+                at = __shfl_sync(kFull, at, 0);
+                if (kn)
+                    s_list[at + (unsigned)__popc(list & ((1u << tx) - 1u))] = (uint16_t)(32 * ly + tx);
+            }
+            if (!kn && in) {
+                for (int ch = 0; ch < C; ++ch) bH[ch * nH + (size_t)Y * wH + X] = 0.f;
+            }
+        }
+    }
+    auto own_values = [&](auto channels) {
+#pragma unroll
+        for (int r = 0; r < R; ++r)
+            if (ck[r]) value(channels, tx, ty + 8 * r, ck[r]);
+    };
+    if (!LIST && !MOD && values) {  // need no neighbours
+        if (C == 1) own_values(std::integral_constant<int, 1>{});
+        else own_values(std::integral_constant<int, kMaxChannels>{});
+    }
+    if (tx == 0) s_unk[ty] = unk;
+    __syncthreads();
+    if (unknown && t == 0) {
+        unsigned a = 0;
+        for (int i = 0; i < 8; ++i) a += s_unk[i];
+        if (a) atomicAdd(unknown, (unsigned long long)a);
+    }
+    if (!values) return;
+    if constexpr (LIST) {
+        const unsigned known = s_n;
+        for (unsigned i = t; i < known; i += 256) {
+            const int e = s_list[i], lx = e & 31, ly = e >> 5;
+            value(std::integral_constant<int, kMaxChannels>{}, lx, ly, s_kn[ly + 1][lx + 1]);
+        }
+    } else if constexpr (MOD) {
+        own_values(std::integral_constant<int, kMaxChannels>{});
     }
 }
 
-template <int R>
+template <int R, bool LIST, bool MOD>
 __global__ void __launch_bounds__(256)
 k_pyramid_level(const uint8_t* __restrict__ c, const float* __restrict__ b, int w, int h, int C,
-                uint8_t* __restrict__ cH, float* __restrict__ bH, int wH, int hH, int modified,
-                int values, uint32_t* __restrict__ bits, int wpr,
+                uint8_t* __restrict__ cH, float* __restrict__ bH, int wH, int hH, int values,
+                uint32_t* __restrict__ bits, int wpr,
                 unsigned long long* __restrict__ unknown) {
-    pyramid_level_body<R>(c, b, w, h, C, cH, bH, wH, hH, modified, values, bits, wpr, unknown,
+    pyramid_level_body<R, LIST, MOD>(c, b, w, h, C, cH, bH, wH, hH, values, bits, wpr, unknown,
                           blockIdx.x, blockIdx.y, gridDim.x);
 }
 
@@ -3386,11 +3409,19 @@ k_batch_grid(const BatchSeg* __restrict__ segs, int nseg, BatchState bs) {
     const int plane = sg.gx * sg.gy;
     const int bz = local / plane, rem = local - bz * plane;
     const int by = rem / sg.gx, bx = rem - by * sg.gx;
-    if (KIND == kBPyramid)
-        pyramid_level_body<1>(static_cast<const uint8_t*>(sg.in0), static_cast<const float*>(sg.in1),
-                           w, h, sg.C, static_cast<uint8_t*>(sg.out0),
-                           static_cast<float*>(sg.out1), wH, hH, sg.mode, 1,
-                           const_cast<uint32_t*>(sg.mbits), sg.wpr, sg.counter, bx, by, sg.gx);
+    if (KIND == kBPyramid) {
+        const uint8_t* c = static_cast<const uint8_t*>(sg.in0);
+        const float* b = static_cast<const float*>(sg.in1);
+        uint8_t* cH = static_cast<uint8_t*>(sg.out0);
+        float* bH = static_cast<float*>(sg.out1);
+        uint32_t* bits = const_cast<uint32_t*>(sg.mbits);
+        if (sg.mode)
+            pyramid_level_body<1, true, true>(c, b, w, h, sg.C, cH, bH, wH, hH, 1, bits, sg.wpr,
+                                              sg.counter, bx, by, sg.gx);
+        else
+            pyramid_level_body<1, false, false>(c, b, w, h, sg.C, cH, bH, wH, hH, 1, bits, sg.wpr,
+                                                sg.counter, bx, by, sg.gx);
+    }
     else if (KIND == kBMaskDown)
         mask_down_body(static_cast<const uint8_t*>(sg.in0), w, h, static_cast<uint8_t*>(sg.out0),
                        wH, hH, bx, by);
@@ -4548,17 +4579,28 @@ cudaError_t launch_pyramid_level(const uint8_t* c, const float* b, int w, int h,
     int wH, hH;
     coarse_dims(w, h, &wH, &hH);
     const int wpr = mask_words_per_row(wH);
-    // one CTA column per packed word of a coarse row but the padding word; four
-    // rows of cells per thread once one row each would take more than one wave
-    // of CTAs (longer lists fill the CTA's threads: at 3840x2160 RGB 22.1 us against
-    // 24.7 with two rows; below, one row each keeps more SMs busy)
+    // one CTA column per packed word of a coarse row but the padding word.  Once
+    // one row of cells per thread would take more than one wave of CTAs: the list
+    // over four rows each (longer lists fill the CTA's threads: at 3840x2160 RGB
+    // 22.1 us against 24.7 with two rows), for the naive average, whose weights
+    // are few instructions, two rows and no list (3840x2160 gray, mask density
+    // 0.04 / 0.9: 16.8 / 18.0 us, with the list 15.8 / 26.7, one row 19.8 / 21.1;
+    // RGB 29.8 / 29.7, 25.6 / 32.8, 31.9 / 31.8).  Smaller levels wait for one
+    // step after the other: one row each and no list (1280x720 RGB at 0.04 / 0.9:
+    // 5.8 / 5.7 us, with the list 7.2 / 7.4).
     const long long one = (long long)(wpr - 1) * ((hH + 7) / 8);
-    if (one > 152 * 6)
-        k_pyramid_level<4><<<dim3((unsigned)(wpr - 1), (unsigned)((hH + 31) / 32)), dim3(32, 8), 0,
-                             s>>>(c, b, w, h, C, cH, bH, wH, hH, modified, values, bits, wpr, unknown);
-    else
-        k_pyramid_level<1><<<dim3((unsigned)(wpr - 1), (unsigned)((hH + 7) / 8)), dim3(32, 8), 0,
-                             s>>>(c, b, w, h, C, cH, bH, wH, hH, modified, values, bits, wpr, unknown);
+    const dim3 blk(32, 8);
+    auto grid = [&](int rows) {
+        return dim3((unsigned)(wpr - 1), (unsigned)((hH + 8 * rows - 1) / (8 * rows)));
+    };
+#define DI_PYRAMID(R, LIST, MOD)                                                                  \
+    k_pyramid_level<R, LIST, MOD><<<grid(R), blk, 0, s>>>(c, b, w, h, C, cH, bH, wH, hH, values, \
+                                                          bits, wpr, unknown)
+    if (one > 152 * 6 && modified) DI_PYRAMID(4, true, true);
+    else if (modified) DI_PYRAMID(1, false, true);
+    else if (one > 152 * 6) DI_PYRAMID(2, false, false);
+    else DI_PYRAMID(1, false, false);
+#undef DI_PYRAMID
     count();
     return cudaGetLastError();
 }

@@ -398,6 +398,21 @@ def test_pyramid_level_large_and_odd(di, h, w):
     assert np.array_equal(N(bH), N(di.values_downsample(T(c), T(fn), T(cH_ref))))
 
 
+@pytest.mark.parametrize("h,w", [(1999, 2003), (1201, 2048), (577, 3333), (700, 1000)])
+@pytest.mark.parametrize("C,modified,density", [(1, False, 0.05), (4, False, 0.6), (1, True, 0.6),
+                                                (4, True, 0.6)])
+def test_pyramid_level_forms(di, h, w, C, modified, density):
+    # the naive average (two rows of cells per thread, one on smaller levels; gray
+    # by itself) and the weights of mostly known cells: the same bits as the
+    # separate steps
+    f, fn, c = _case(h, w, C, density, h + w + C)
+    cH, bH, _, unk = di.pyramid_level(T(c), T(fn), modified=modified)
+    cH_ref = M.mask_downsample(c)
+    assert np.array_equal(N(cH), cH_ref) and int(N(unk)[0]) == int((cH_ref == 0).sum())
+    assert np.array_equal(N(bH), N(di.values_downsample(T(c), T(fn), T(cH_ref),
+                                                        modified=modified)))
+
+
 @pytest.mark.parametrize("C", [2, 3, 4])
 @pytest.mark.parametrize("h,w,aligned", [(1200, 1100, True), (1101, 1203, True), (1200, 1100, False)])
 @pytest.mark.parametrize("rhs_zero", [True, False])
