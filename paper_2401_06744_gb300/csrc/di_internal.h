@@ -101,6 +101,11 @@ inline size_t oras_scratch_floats(int w, int h, int C, int B, int o) {
     return (size_t)axis_blocks_decl(w, B, o) * axis_blocks_decl(h, B, o) * C * B * B;
 }
 
+// Local problems (blocks x channels) of a launch up to which 32x32 blocks with
+// FP32 iterates, an even overlap and FP32 residuals take four warps per problem
+// instead of two (the same bits); the tests look up which form they reach.
+int oras_quad_tasks();
+
 // One ORAS iteration u_in -> u_out (parked: oras_scratch_floats of workspace;
 // mbits: the packed mask of this level).  Each local CG runs `iters` steps or
 // until r.r <= max(rtol2, 1e-14) * (r.r)_0 (rtol2 >= 0), or until

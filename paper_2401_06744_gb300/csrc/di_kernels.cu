@@ -3936,7 +3936,7 @@ const void* oras_2w_h_fn() {
 }
 
 // Local problems of a launch up to which the four-warp form takes it: four per
-// SM, what is resident at once (at 80 registers for six, the 256x256 decode took
+// SM of the 152, what is resident at once (at 80 registers for six, the 256x256 decode took
 // 218 us instead of 211).
 // Decodes of 256x256 / 481x321 RGB / 1920x1080 RGB with the line at 0, 1, 2, 4
 // and 6 per SM: 249, 212, 212, 211, 211 / 432, 404, 396, 394, 393 / 1115, 1094,
@@ -4441,6 +4441,8 @@ cudaError_t launch_wait_selftest(unsigned* flag, int limit, cudaStream_t s) {
     count();
     return cudaGetLastError();
 }
+
+int oras_quad_tasks() { return kQuadTasks; }
 
 cudaError_t launch_pack_mask(const uint8_t* c, int w, int h, uint32_t* bits,
                              unsigned long long* unknown, cudaStream_t s) {

@@ -7,6 +7,8 @@ operation on such values carries an error of about 255 * 2^-24 = 1.5e-5, so
 stencil-sized expressions are compared at 2e-4 (absolute) and the ORAS
 iteration, whose local PCG amplifies rounding over its steps, at 1e-3 of the
 largest correction plus 2e-4."""
+import ctypes
+
 import numpy as np
 import pytest
 import torch
@@ -303,8 +305,20 @@ def test_oras_shared_pixels_of_small_blocks(di, h, w, B, o):
     assert np.abs(out - ref).max() < 1e-3 * np.abs(ref - u).max() + 2e-4
 
 
+def _quad_tasks(di):
+    # local problems up to which a launch takes four warps per problem
+    fn = ctypes.CDLL(di.LIB_PATH)["_ZN2di15oras_quad_tasksEv"]
+    fn.restype = ctypes.c_int
+    return fn()
+
+
+def _blocks(h, w, o):
+    return len(M.axis_blocks(h, 32, o)) * len(M.axis_blocks(w, 32, o))
+
+
 QUAD_CASES = [  # (h, w, overlap, aligned): up to 608 local problems in one channel, more in four
     (601, 600, 2, True), (500, 601, 6, True), (601, 640, 4, False), (660, 580, 2, False),
+    (601, 600, 4, True), (487, 604, 6, True), (481, 320, 16, True),
 ]
 
 
@@ -314,6 +328,7 @@ def test_oras_few_problems_same_bits(di, h, w, o, aligned, rhs_zero):
     # launches of few local problems take four warps per problem, larger ones two:
     # one channel alone and the same channel among four give the same bits, for
     # the plain iteration and both prolonged starts
+    assert _blocks(h, w, o) <= _quad_tasks(di) < 4 * _blocks(h, w, o)
     f, fn, c = _case(h, w, 1, 0.06, h + 3 * w + o)
     g = np.random.default_rng(w)
     H, W = M.coarse_shape(h, w)
@@ -364,6 +379,72 @@ def test_oras_of_a_scaled_image(di, C, o, rhs_zero):
             k = np.float32(2.0 ** e)
             out = N(ctx.oras_iteration(T(u * k), T(b * k), T(c), 12, rhs_zero=rhs_zero))
             assert np.array_equal(out, ref * k), e
+
+
+TWO_WARP_CASES = [  # (h, w, overlap, aligned): last blocks of different heights and widths
+    (480, 640, 2, True), (453, 640, 2, False), (461, 641, 2, True), (480, 640, 4, True),
+    (437, 652, 4, True), (461, 640, 4, False), (480, 640, 6, True), (431, 604, 6, True),
+    (449, 607, 6, True), (453, 600, 6, False), (300, 404, 16, True),
+]
+
+
+@pytest.mark.parametrize("h,w,o,aligned", TWO_WARP_CASES)
+@pytest.mark.parametrize("rhs_zero", [True, False])
+def test_oras_two_warps_per_problem(di, h, w, o, aligned, rhs_zero):
+    # launches of more local problems than take four warps each, through TMA tiles
+    # (aligned, w a multiple of 4) and cp.async: the iteration against the oracle's
+    # (the bounds of test_oras_iteration_matches_oracle_cg) and both prolonged
+    # starts against their two steps (identical bits)
+    C, K = 3, 6
+    assert C * _blocks(h, w, o) > _quad_tasks(di)
+    f, fn, c = _case(h, w, C, 0.06, h + 5 * w + o)
+    g = np.random.default_rng(3 * h + w)
+    H, W = M.coarse_shape(h, w)
+    known = c.astype(bool)
+    if rhs_zero:
+        u = np.where(known, f, g.uniform(0, 255, f.shape)).astype(np.float32)
+        b, ref_b, atol = fn, M.rhs(f, c), 2e-4
+    else:
+        u = np.where(known, 0.0, g.normal(size=f.shape)).astype(np.float32)
+        b = np.where(known, 0.0, g.normal(size=f.shape)).astype(np.float32)
+        ref_b, atol = b, 1e-5
+    uH = g.normal(scale=4.0, size=(C, H, W)).astype(np.float32)
+    put = T if aligned else _unaligned
+    with di.Context(block=32, overlap=o, alpha=0.4) as ctx:
+        out = N(ctx.oras_iteration(put(u), put(b), T(c), K, rhs_zero=rhs_zero))
+        ref = M.oras_iteration(u, ref_b, c, 32, o, 0.4, ("cg", K))
+        assert np.abs(out - ref).max() < 1e-3 * np.abs(ref - u).max() + atol
+        up = put(u)
+        di.prolong(T(uH), T(c), 1, u=up)
+        two = N(ctx.oras_iteration(up, put(b), T(c), K, rhs_zero=rhs_zero))
+        fused = N(ctx.prolong_oras_iteration(T(uH), put(u), put(b), T(c), K, rhs_zero=rhs_zero))
+        assert np.array_equal(fused, two)
+        if rhs_zero:
+            start = di.prolong(T(uH), T(c), 0, b=put(fn))
+            two = N(ctx.oras_iteration(start, put(fn), T(c), K, rhs_zero=True))
+            fused = N(ctx.prolong_oras_iteration(T(uH), put(fn), put(fn), T(c), K, rhs_zero=True,
+                                                 mode=0))
+            assert np.array_equal(fused, two)
+
+
+@pytest.mark.parametrize("o", [1, 2, 5, 6, 16])
+@pytest.mark.parametrize("h,w", [(77, 96), (62, 95)])
+def test_oras_fp64_residual_steps(di, h, w, o):
+    # FP64 block residuals at even and odd overlaps, with and without a right-hand
+    # side: the bounds of test_oras_iteration_matches_oracle_cg
+    f, fn, c = _case(h, w, 2, 0.07, h + w + o)
+    g = np.random.default_rng(o)
+    known = c.astype(bool)
+    u = np.where(known, f, g.uniform(0, 255, f.shape)).astype(np.float32)
+    e = np.where(known, 0.0, g.normal(size=f.shape)).astype(np.float32)
+    b = np.where(known, 0.0, g.normal(size=f.shape)).astype(np.float32)
+    with di.Context(block=32, overlap=o, alpha=0.4, refine_fp64=1) as ctx:
+        out = N(ctx.oras_iteration(T(u), T(fn), T(c), 6, rhs_zero=True))
+        ref = M.oras_iteration(u, M.rhs(f, c), c, 32, o, 0.4, ("cg", 6))
+        assert np.abs(out - ref).max() < 1e-3 * np.abs(ref - u).max() + 2e-4
+        out = N(ctx.oras_iteration(T(e), T(b), T(c), 6, rhs_zero=False))
+        ref = M.oras_iteration(e, b, c, 32, o, 0.4, ("cg", 6))
+        assert np.abs(out - ref).max() < 1e-3 * np.abs(ref - e).max() + 1e-5
 
 
 @pytest.mark.parametrize("w", [16, 48, 64, 112, 4112])
