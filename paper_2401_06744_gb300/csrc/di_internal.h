@@ -225,24 +225,24 @@ enum BatchWhen {
 };
 
 enum BatchKind {  // grid kernels of the batched form
-    kBMaskDown = 0, kBValuesDown = 1, kBPack = 2, kBSelect = 3, kBRestrict = 4, kBProlong = 5,
-    kBPyramid = 6  // one pyramid level in one pass (mask, values, packed words, unknown count)
+    kBPack = 0, kBSelect = 1, kBRestrict = 2,
+    kBPyramid = 3  // one pyramid level in one pass (mask, values, packed words, unknown count)
 };
 
 struct BatchSeg {
     int first;             // first CTA (grid kernels) or block unit (block kernel)
     int gx, gy;            // grid kernels: CTAs along x and y per channel plane
-    int w, h, C;           // level size (the fine level for restriction and prolongation)
+    int w, h, C;           // level size (the fine level for pyramid level and restriction)
     int img, level, when;  // image, level and participation (BatchWhen)
     int L;                 // the image's pyramid depth
-    const void* in0;       // mask_down, values_down, pack: c; restrict: u; prolong: uH; block: u_in
-    const void* in1;       // values_down: b; select: b; restrict: b; prolong: b; block: rhs
-    const void* in2;       // values_down: cH; select: c; restrict: cH; prolong: c
-    void* out0;            // mask_down: cH; values_down: bH; select: u; restrict: rH; prolong, block: u
-    void* out1;            // select: a second u written alike (nullable)
-    const uint32_t* mbits; // pack: bits out; block: the level's packed mask
-    unsigned* maxupd;      // prolong, block: the image's update slot (nullable)
-    unsigned long long* counter;  // pack: the image's unknown count of this level
+    const void* in0;       // pack, pyramid: c; restrict: u; block: u_in
+    const void* in1;       // pyramid, select, restrict: b; block: rhs
+    const void* in2;       // select: c; restrict: cH
+    void* out0;            // pyramid: cH; select, block: u; restrict: rH
+    void* out1;            // pyramid: bH; select: a second u written alike (nullable)
+    const uint32_t* mbits; // pack, pyramid: bits out; block: the level's packed mask
+    unsigned* maxupd;      // block: the image's update slot (nullable)
+    unsigned long long* counter;  // pack, pyramid: the image's unknown count of this level
     int zero_in, rhs_zero, iters, nbx, nby, wpr, mode, keep;  // zero_in: one value per launch
     float rtol2;
     // block kernel: the start prolonged from the next coarser level inside the

@@ -3424,15 +3424,7 @@ k_batch_grid(const BatchSeg* __restrict__ segs, int nseg, BatchState bs) {
         else
             pyramid_level_body<1, false, false>(c, b, w, h, sg.C, cH, bH, wH, hH, 1, bits, sg.wpr,
                                                 sg.counter, bx, by, sg.gx);
-    }
-    else if (KIND == kBMaskDown)
-        mask_down_body(static_cast<const uint8_t*>(sg.in0), w, h, static_cast<uint8_t*>(sg.out0),
-                       wH, hH, bx, by);
-    else if (KIND == kBValuesDown)
-        values_down_body(static_cast<const uint8_t*>(sg.in0), static_cast<const float*>(sg.in1),
-                         w, h, sg.C, static_cast<const uint8_t*>(sg.in2),
-                         static_cast<float*>(sg.out0), wH, hH, sg.mode, bx, by);
-    else if (KIND == kBRestrict) {
+    } else if (KIND == kBRestrict) {
         const float* u = static_cast<const float*>(sg.in0);
         const float* b = static_cast<const float*>(sg.in1);
         const uint8_t* cH = static_cast<const uint8_t*>(sg.in2);
@@ -3445,12 +3437,6 @@ k_batch_grid(const BatchSeg* __restrict__ segs, int nseg, BatchState bs) {
             restrict_body<false, float, float, float, false>(u, b, sg.rhs_zero, w, h, cH, rH, wH,
                                                              hH, bx, by, bz);
     }
-    else if (KIND == kBProlong)
-        prolong_body<false, float, float>(static_cast<const float*>(sg.in0), wH, hH,
-                                          static_cast<const float*>(sg.in1),
-                                          static_cast<const uint8_t*>(sg.in2), w, h,
-                                          static_cast<float*>(sg.out0), sg.mode, sg.maxupd, bx,
-                                          by, bz);
 }
 
 // The block kernel over the block units of a batch: a unit is one 32x32
@@ -4514,8 +4500,7 @@ void batch_grid_dims(int kind, int w, int h, int* gx, int* gy) {
         if (b > 1024) b = 1024;
         *gx = (int)(b < 1 ? 1 : b);
         *gy = 1;
-    } else if (kind == kBRestrict || kind == kBProlong || kind == kBMaskDown ||
-               kind == kBValuesDown || kind == kBPyramid) {  // a coarse cell per thread, 32 x 8 per CTA
+    } else if (kind == kBRestrict || kind == kBPyramid) {  // a coarse cell per thread, 32 x 8 per CTA
         const int wH = (w + 1) / 2, hH = (h + 1) / 2;
         *gx = (wH + 31) / 32;
         *gy = (hH + 7) / 8;
@@ -4529,12 +4514,9 @@ cudaError_t launch_batch_grid(int kind, const BatchSeg* segs, int nseg, int ncta
     if (nctas < 1 || nseg < 1) return cudaSuccess;
     const dim3 blk2(32, 8), blk1(256);
     switch (kind) {
-        case kBMaskDown: k_batch_grid<kBMaskDown><<<nctas, blk2, 0, s>>>(segs, nseg, bs); break;
-        case kBValuesDown: k_batch_grid<kBValuesDown><<<nctas, blk2, 0, s>>>(segs, nseg, bs); break;
         case kBPack: k_batch_grid<kBPack><<<nctas, blk1, 0, s>>>(segs, nseg, bs); break;
         case kBSelect: k_batch_grid<kBSelect><<<nctas, blk1, 0, s>>>(segs, nseg, bs); break;
         case kBRestrict: k_batch_grid<kBRestrict><<<nctas, blk2, 0, s>>>(segs, nseg, bs); break;
-        case kBProlong: k_batch_grid<kBProlong><<<nctas, blk2, 0, s>>>(segs, nseg, bs); break;
         case kBPyramid: k_batch_grid<kBPyramid><<<nctas, blk2, 0, s>>>(segs, nseg, bs); break;
         default: return cudaErrorInvalidValue;
     }
