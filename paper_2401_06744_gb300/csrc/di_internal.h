@@ -157,7 +157,8 @@ cudaError_t launch_cg_smooth(const float* in, int zero_in, const float* b, int r
 // whole decode runs as one CUDA graph without host round trips.
 // ---------------------------------------------------------------------------
 
-// Stop-test state of one decode (device memory, read back once at the end).
+// Stop-test state of one decode (device memory; the plan and the stop test that
+// ends it write it to a pinned host copy).
 struct StopState {
     int cycles;          // V-cycles run
     int status;          // di_status of the decode

@@ -7,12 +7,15 @@
 // Kernels:
 //   k_pyramid_level  Section 4.3: one pyramid level in one pass (2x2 max pooling of
 //                    the mask, modified or naive mask values, packed mask words,
-//                    unknown count); k_mask_down, k_values_down and k_pack_mask
-//                    are the separate steps (single-step entry points, the finest
-//                    level's packing)
+//                    unknown count); k_mask_down and k_values_down are the
+//                    separate steps of the single-step entry points
+//   k_pack_mask16    the finest level's packed mask words and unknown count, 16 mask
+//                    bytes per thread; k_pack_mask for rows of other widths
 //   k_residual       r = b - A u with per-CTA partial sums of r^2 (Algorithm 2 step 1)
 //   k_reduce         fixed-order sum of the partials (one global scalar product)
-//   k_restrict       Algorithm 3 steps 2-3 fused: residual + 2x2 averaging (x4)
+//   k_restrict       Algorithm 3 steps 2-3 fused: residual + 2x2 averaging (x4);
+//                    k_restrict_c for the large levels of FP32 images (every
+//                    channel of a cell by one thread)
 //   k_prolong        Section 4.4 bilinear prolongation, cascadic or correction mode
 //                    (where the block kernel cannot form its start by prolongation)
 //   k_select         u = c ? b : 0 (or c ? b : u for a given start)
@@ -1483,8 +1486,8 @@ struct Smem2W {
 // lane shuffles per warp and CG step, where the lane = column layout took 42
 // and where shuffles and shared-memory accesses share one pipe.  Tile loads and
 // the write of u are 8-byte words.  4K RGB, overlap 2: 13.6 us per CG step
-// (lane = column layout: 16.0), 178 warp instructions per warp and step (221); a
-// task without steps 598 (706).
+// (lane = column layout: 16.0), 176 warp instructions per warp and step (221); a
+// task without steps 612 (706), 937 with the prolongation.
 struct BlockThread {
     int lane, wi, g, l;
     int cl;      // first of the two columns
@@ -2066,10 +2069,10 @@ __device__ __forceinline__ void tma_load_3d(unsigned dst, const CUtensorMap* map
 // the known pixels and P eH at the unknown ones (prolong_body's mode 0 with
 // u_in as b: the cascade's interpolation of the coarser level's solution).
 // Each block forms the start in its tile (block pixels and halo) before the
-// residual.  OV: 0 overlap 2 (partition weights 0 and 1); blocks share pixels
-// (overlap 1 or >= 3) and 1 the block stride 32 - o is even, 2 odd (block
-// columns at odd pixels: no 8-byte words).  Needs u_in (not zero_in) and an even block stride, so that the
-// parity of a block pixel is that of its tile index.
+// residual.  PRO needs u_in (not zero_in) and an even block stride, so that the
+// parity of a block pixel is that of its tile index.  OV: 0 overlap 2 (partition
+// weights 0 and 1); blocks share pixels (overlap 1 or >= 3) and 1 the block
+// stride 32 - o is even, 2 odd (block columns at odd pixels: no 8-byte words).
 template <bool F64, int PRO, int OV>
 __global__ void __launch_bounds__(64, 8)
 k_oras_2w(const float* __restrict__ u_in, int zero_in, const float* __restrict__ rhs,
@@ -3701,7 +3704,8 @@ k_batch_oras(const BatchSeg* __restrict__ segs, int nseg, int nunits, int split,
 // The same with four warps per local problem (oras_4w), for launches of few:
 // CTA cmax * g + ch takes channel ch of block unit g.  With it, and the
 // channels of a block on separate CTAs where there are fewer blocks than CTA
-// slots, a batch of 12 images of 640x481 went from 1340 to 1167 us.
+// slots, a batch of 12 uneven images up to 1920x1080 takes 1077 us instead of
+// 1272, two cycles of 12 RGB and gray images of 640x481 984 instead of 1189.
 __global__ void __launch_bounds__(128, 4)
 k_batch_oras_4w(const BatchSeg* __restrict__ segs, int nseg, int cmax, int o, float alpha,
                 BatchState bs) {
