@@ -3432,6 +3432,9 @@ k_batch_grid(const BatchSeg* __restrict__ segs, int nseg, BatchState bs) {
         const float* b = static_cast<const float*>(sg.in1);
         const uint8_t* cH = static_cast<const uint8_t*>(sg.in2);
         float* rH = static_cast<float*>(sg.out0);
+        // patches beside the mask bytes: whole batches are 1 % faster for it at a
+        // mask density of 0.05 and 2 % slower at 0.9 (eight images of 1920x1080:
+        // 2774 against 2799 us, 2054 against 2018)
         if ((w & 1) == 0 && ((reinterpret_cast<uintptr_t>(u) |
                               (sg.rhs_zero ? 0 : reinterpret_cast<uintptr_t>(b))) & 7) == 0)
             restrict_body<true, float, float, float, false, true>(u, b, sg.rhs_zero, w, h, cH, rH,
